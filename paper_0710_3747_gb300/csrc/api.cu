@@ -476,6 +476,10 @@ static int init_blocks(int M) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(n, 152 * 8));
 }
 
+// Blocks of init_kernel (half as many: its FP64 reduction costs each thread
+// about ten FP64 additions, whatever the thread's share of the state).
+static int fill_blocks(int M) { return std::min(init_blocks(M), 152 * 4); }
+
 // Build the sweep descriptors for plan p.
 static void build_passes(const Plan &p, bool has_diag, PassSet *ps) {
   const int M = p.M, K = p.K, c = p.c;
@@ -1219,15 +1223,16 @@ static int record_sites0(spinrp_state *st) {
 static int state_init(spinrp_state *st, uint64_t seed, int kind) {
   if (!st) return fail(SPINRP_EINVAL, "init: state is NULL");
   begin_series(st);
-  const int blocks = init_blocks(st->M);
+  const int blocks = fill_blocks(st->M);
+  const double amp = std::exp2(-0.5 * (st->M - 1));
   prof_mark(st, SPINRP_KERNEL_INIT);
   ++g_launches;
   if (st->prec == SPINRP_C64)
-    init_kernel<float><<<blocks, 256, 0, st->stream>>>(st->d_job, st->M, layout_arg(st), seed, nullptr,
-                                                       kind, st->orient_black);
+    init_kernel<float><<<blocks, 256, 0, st->stream>>>(st->d_job, st->M, layout_arg(st), amp, st->plan.pos[0], seed,
+                                                       nullptr, kind, st->orient_black);
   else
-    init_kernel<double><<<blocks, 256, 0, st->stream>>>(st->d_job, st->M, layout_arg(st), seed, nullptr,
-                                                        kind, st->orient_black);
+    init_kernel<double><<<blocks, 256, 0, st->stream>>>(st->d_job, st->M, layout_arg(st), amp, st->plan.pos[0], seed,
+                                                        nullptr, kind, st->orient_black);
   CUDA_TRY(cudaGetLastError());
   int rc = record_sites0(st);
   if (rc) return rc;
@@ -2747,13 +2752,15 @@ static LayoutArg group_layout(const BatchGroup &g) {
 static int batch_init(spinrp_batch *b, int kind) {
   if (!b) return fail(SPINRP_EINVAL, "batch_init: batch is NULL");
   for (BatchGroup &g : b->groups) {
-    const dim3 grid(init_blocks(g.M), (unsigned)g.jobs.size());
+    const dim3 grid(fill_blocks(g.M), (unsigned)g.jobs.size());
+    const double amp = std::exp2(-0.5 * (g.M - 1));
     ++g_launches;
     if (b->prec == SPINRP_C64)
-      init_kernel<float><<<grid, 256, 0, b->stream>>>(g.d_jobs, g.M, group_layout(g), 0, g.d_seeds, kind,
-                                                      g.ps.oriented ? g.ps.black : 0ull);
+      init_kernel<float><<<grid, 256, 0, b->stream>>>(g.d_jobs, g.M, group_layout(g), amp, g.plan.pos[0], 0,
+                                                      g.d_seeds, kind, g.ps.oriented ? g.ps.black : 0ull);
     else
-      init_kernel<double><<<grid, 256, 0, b->stream>>>(g.d_jobs, g.M, group_layout(g), 0, g.d_seeds, kind, 0);
+      init_kernel<double><<<grid, 256, 0, b->stream>>>(g.d_jobs, g.M, group_layout(g), amp, g.plan.pos[0], 0,
+                                                       g.d_seeds, kind, 0);
     CUDA_TRY(cudaGetLastError());
   }
   b->len = 1;

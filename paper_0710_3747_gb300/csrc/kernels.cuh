@@ -255,18 +255,20 @@ sites_finalize_kernel(const JobPtrs *__restrict__ jobs, int M, int nblk) {
 // fixed-point turns.
 enum InitKind { INIT_ENTANGLED = 0, INIT_PRODUCT = 1 };
 
+// amp_d: 2^{-(M-1)/2}, p0: the physical position of spin 1 (both from the
+// host: a double exp2 in every thread cost 15 us by itself, FP64 runs at 1/64
+// of the FP32 rate).
 // orient: logical mask of the first-colour spins of an oriented state (0 for
 // a plain one): amplitudes with an odd number of them up are stored (Im, Re).
 template <typename R>
 __global__ void __launch_bounds__(256)
-init_kernel(const JobPtrs *__restrict__ jobs, int M, LayoutArg lay, uint64_t seed0,
-            const uint64_t *__restrict__ seeds, int kind, uint64_t orient) {
+init_kernel(const JobPtrs *__restrict__ jobs, int M, const __grid_constant__ LayoutArg lay, double amp_d, int p0,
+            uint64_t seed0, const uint64_t *__restrict__ seeds, int kind, uint64_t orient) {
   using C = typename CT<R>::T;
   const JobPtrs jp = jobs[blockIdx.y];
   C *__restrict__ psi = static_cast<C *>(jp.psi);
   const uint64_t seed = seeds ? seeds[blockIdx.y] : seed0;
-  const uint64_t N = 1ull << M;
-  const R amp = (R)exp2(-0.5 * (double)(M - 1));
+  const R amp = (R)amp_d;
   const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
   // product state: turns u_l * 2^64 of each physical bit position (0 for spin 1)
   __shared__ uint64_t s_turns[kMaxM];
@@ -282,45 +284,88 @@ init_kernel(const JobPtrs *__restrict__ jobs, int M, LayoutArg lay, uint64_t see
     }
     __syncthreads();
   }
-  R up = 0, dn = 0;
-  for (uint64_t y = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; y < N;
-       y += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t x = 0;
-    for (int p = 0; p < M; ++p) x |= ((y >> p) & 1ull) << lay.logical_of[p];
-    C v;
-    if ((x & 1ull) == 0) {
-      v.x = 0, v.y = 0;
-    } else if (kind == INIT_PRODUCT) {
-      uint64_t th = 0;
-      for (int p = 0; p < M; ++p)
-        if ((y >> p) & 1ull) th -= s_turns[p];
-      const C e = cis_turns(th, (R)0);
-      v.x = amp * e.x, v.y = amp * e.y;
-      up += v.x * v.x + v.y * v.y;
-    } else {
-      const uint64_t r = x >> 1;
-      const uint4 w = philox4x32_10(make_uint4((uint32_t)r, (uint32_t)(r >> 32), 0u, 0u), key);
-      const uint64_t bits = ((uint64_t)w.x << 32) | w.y;
-      C e;
-      if (sizeof(R) == 8) {
-        // u = top 53 bits * 2^-53 exactly as defined; angle 2 pi u
-        double s, c;
-        sincospi(2.0 * ((double)(bits >> 11) * 1.1102230246251565e-16), &s, &c);
-        e.x = (R)c, e.y = (R)s;
-      } else {
-        const float2 f = cis_turns(bits, 0.0f);
-        e.x = (R)f.x, e.y = (R)f.y;
-      }
-      v.x = amp * e.x, v.y = amp * e.y;
-      up += v.x * v.x + v.y * v.y;
+  // Index z runs over the 2^(M-1) basis states with spin 1 up, physical bits
+  // without spin 1's position p0; its partner with spin 1 down is zero and
+  // written beside it.  Bits 0..7 of z come from the thread, the next eb from a
+  // loop, the rest from the chunk the block takes, and z's logical index (and
+  // product phase) is a sum over its bits, so each group of bits is summed once
+  // where it changes.  Bound by Philox and sincos (about 130 instructions a
+  // state) next to the store: mapping the bits one by one for every amplitude
+  // took twelve times the store's time (complex64, 2^26 amplitudes: 948 us before,
+  // 241 us so, 79 us for the store alone; 2^20: 29 us before, 16 us so).
+  const int n = M - 1, eb = min(4, max(0, n - 18)), lane = threadIdx.x & 31;
+  auto phys = [&](int k) { return k < p0 ? k : k + 1; };  // physical position of bit k of z
+  uint64_t x_thr = 1, th_thr = 0;
+  for (int k = 0; k < 8 && k < n; ++k)
+    if ((threadIdx.x >> k) & 1) {
+      x_thr |= 1ull << lay.logical_of[phys(k)];
+      if (kind == INIT_PRODUCT) th_thr -= s_turns[phys(k)];
     }
-    if (__popcll(x & orient) & 1) {
-      const R t = v.x;
-      v.x = v.y, v.y = t;
-    }
-    psi[y] = v;
+  // the loop's bits: one mask (and product phase) each
+  uint64_t x_e[4], th_e[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    x_e[k] = k < eb ? 1ull << lay.logical_of[phys(8 + k)] : 0ull;
+    th_e[k] = kind == INIT_PRODUCT && k < eb ? s_turns[phys(8 + k)] : 0ull;
   }
-  reduce_finalize((double)up, (double)dn, jp, true);
+  const uint64_t chunks = n > 8 + eb ? 1ull << (n - 8 - eb) : 1ull, low = (1ull << p0) - 1ull;
+  double up = 0;
+  for (uint64_t c = blockIdx.x; c < chunks; c += gridDim.x) {
+    // the chunk's bits: lane k has bit 8 + eb + k (fewer than 32)
+    const int kc = 8 + eb + lane;
+    const bool on = kc < n && ((c >> lane) & 1ull);
+    const uint64_t xb = on ? 1ull << lay.logical_of[phys(kc)] : 0ull;
+    uint64_t th_c = th_thr;
+    if (kind == INIT_PRODUCT) {
+      uint64_t t = on ? s_turns[phys(kc)] : 0ull;
+      for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      th_c -= t;
+    }
+    const uint64_t x_c = x_thr | __reduce_or_sync(0xffffffffu, (uint32_t)xb) |
+                         (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(xb >> 32)) << 32;
+    R part = 0;
+#pragma unroll 2
+    for (int e = 0; e < (1 << eb); ++e) {
+      const uint64_t z = (((c << eb) | (uint64_t)e) << 8) | threadIdx.x;
+      if (z >= 1ull << n) break;
+      uint64_t x = x_c, th = th_c;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if ((e >> k) & 1) x |= x_e[k], th -= th_e[k];
+      C v;
+      if (kind == INIT_PRODUCT) {
+        const C t = cis_turns(th, (R)0);
+        v.x = amp * t.x, v.y = amp * t.y;
+      } else {
+        const uint64_t r = x >> 1;
+        const uint4 w = philox4x32_10(make_uint4((uint32_t)r, (uint32_t)(r >> 32), 0u, 0u), key);
+        const uint64_t bits = ((uint64_t)w.x << 32) | w.y;
+        C t;
+        if (sizeof(R) == 8) {
+          // u = top 53 bits * 2^-53 exactly as defined; angle 2 pi u
+          double s, cc;
+          sincospi(2.0 * ((double)(bits >> 11) * 1.1102230246251565e-16), &s, &cc);
+          t.x = (R)cc, t.y = (R)s;
+        } else {
+          const float2 f = cis_turns(bits, 0.0f);
+          t.x = (R)f.x, t.y = (R)f.y;
+        }
+        v.x = amp * t.x, v.y = amp * t.y;
+      }
+      part += v.x * v.x + v.y * v.y;
+      if (__popcll(x & orient) & 1) {
+        const R t = v.x;
+        v.x = v.y, v.y = t;
+      }
+      const uint64_t y = ((z & ~low) << 1) | (z & low);
+      C zero;
+      zero.x = 0, zero.y = 0;
+      psi[y] = zero;
+      psi[y | (low + 1ull)] = v;
+    }
+    up += (double)part;
+  }
+  reduce_finalize(up, 0.0, jp, true);
 }
 
 // ---------------------------------------------------------------------------
