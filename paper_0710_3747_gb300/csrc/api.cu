@@ -392,11 +392,18 @@ struct PassSet {
   int rb = 5;           // their register bits per phase
   bool oriented = false;  // the programs are oriented (and so is the state)
   uint64_t black = 0;     // first-colour spins (logical mask) when oriented
+  DiagTab tab;            // tables of the diagonal op
+  // pipe_kernel's variant for a pass: with the diagonal op; else by its gates
+  // per phase (a walk over the register-bit pairs pays from kPipeDenseGates on)
+  int variant(int pass) const {
+    const PassDesc &d = desc[pass];
+    return d.diag >= 0 ? kPipeDiag : d.nops >= kPipeDenseGates * d.nphases ? kPipeDense : kPipeSparse;
+  }
 };
 
 struct Layout {  // byte offsets inside the work buffer
   size_t series, partials, ticket, job, coefs, bvals, adiag, qdiag, passes, ops, phases, rops, stage,
-      stage_idx, psites, site_series, sops, total;
+      stage_idx, psites, site_series, sops, dtab, total;
 };
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -503,6 +510,7 @@ static void build_passes(const Plan &p, bool has_diag, PassSet *ps) {
     std::vector<int> in_spin(M, -1), out_spin(M, -1);  // physical position -> spin
     for (int q = 0; q < M; ++q) in_spin[Lin[q]] = q, out_spin[Lout[q]] = q;
     d.relabel = 0;
+    d.diag = -1;
     for (int qo = 0; qo < K; ++qo) {
       d.tile_pos[qo] = (uint8_t)tpos[qo];
       const int spin = out_spin[tpos[qo]];
@@ -548,6 +556,7 @@ static void build_passes(const Plan &p, bool has_diag, PassSet *ps) {
     op.kind = OP_DIAG;
     op.arg = (uint8_t)variant;
     push(pass, op);
+    ps->desc[pass].diag = variant;
   };
   auto reduce = [&](int pass) {
     Op op{};
@@ -589,15 +598,10 @@ static void build_passes(const Plan &p, bool has_diag, PassSet *ps) {
     std::vector<int> spin_at(M);
     for (int q = 0; q < M; ++q) spin_at[out[q]] = q;
     const std::vector<int> &X = p.exitX[k];
-    for (int x : X) {
-      if (out[x] < c) continue;
-      for (int pl = 0; pl < c; ++pl) {
-        const int y = spin_at[pl];
-        if (std::find(X.begin(), X.end(), y) != X.end()) continue;
-        std::swap(out[x], out[y]);
-        spin_at[out[x]] = x, spin_at[out[y]] = y;
-        break;
-      }
+    for (int pl = 0; pl < (int)X.size(); ++pl) {
+      const int x = X[pl], y = spin_at[pl];
+      std::swap(out[x], out[y]);
+      spin_at[out[x]] = x, spin_at[out[y]] = y;
     }
     L[k] = out;
     const int id = new_pass(k, L[k - 1], L[k]);
@@ -635,6 +639,7 @@ static Layout work_layout(int M, int nb, int64_t cap, const PassSet &ps, int max
   L.psites = o, o = align256(o + sizeof(double) * (M + 1) * (size_t)max_blocks);
   L.site_series = o, o = align256(o + sizeof(double) * M * (size_t)std::max<int64_t>(cap, 1));
   L.sops = o, o = align256(o + sizeof(ROpRes) * std::max<size_t>(ps.rops.size(), 1));
+  L.dtab = o, o = align256(o + sizeof(uint64_t) * 2 * ps.tab.words);
   L.total = o;
   return L;
 }
@@ -661,194 +666,293 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
                            bool oriented = false, uint64_t black = 0) {
   ps->phases.clear();
   ps->rops.clear();
+  ps->tab = DiagTab{};
+  const bool rounds = prec == SPINRP_C64 && !oriented;  // the plain complex64 kernels' programs
   const bool wide = prec != SPINRP_C64;  // 16-byte amplitudes, swizzle_slot16
   auto slot_of = [&](uint32_t t) { return wide ? swizzle_slot16(t) : swizzle_slot(t); };
   // lane bits of distinct residues mod `nres` give an access group distinct
   // banks: four (mod 4) for 8-byte amplitudes, three (mod 3) for 16-byte ones
   const int nres = wide ? 3 : 4;
   for (PassDesc &d : ps->desc) {
-    // store order: chunk-index bits 0..2 are output bits 1..3 (128-byte runs);
-    // the fourth, the last lane bit of a half-warp, is the output bit whose
-    // input bit completes four distinct slot residues, so the half-warp's
-    // 8-byte gathers from the tile hit 16 distinct bank pairs
+    // store order: chunk-index bits 0..3, a half-warp's lane bits, are output
+    // bits, the lowest first, whose input bits have independent slot nibbles
+    // (so the half-warp's 8-byte gathers from the tile hit 16 distinct bank
+    // pairs); then the low bits left out, so that a warp still fills 128-byte
+    // lines, then the others
     {
-      auto nib = [&](int q) { return swizzle_slot(1u << d.perm[q]) & 15u; };
-      std::vector<int> order = {1, 2, 3};
-      int pick = -1;
-      for (int x = 4; x < K && pick < 0; ++x) {
-        const uint32_t a = nib(1), b = nib(2), c = nib(3), e = nib(x);
-        // independence of the four nibbles over GF(2)
-        bool indep = true;
-        for (int m = 1; m < 16 && indep; ++m) {
-          const uint32_t v = ((m & 1) ? a : 0u) ^ ((m & 2) ? b : 0u) ^ ((m & 4) ? c : 0u) ^ ((m & 8) ? e : 0u);
-          if (v == 0u) indep = false;
+      std::vector<int> order, rest;
+      std::vector<uint32_t> span = {0u};
+      for (int x = 1; x < K; ++x) {
+        const uint32_t nib = swizzle_slot(1u << d.perm[x]) & 15u;
+        if (order.size() < 4 && std::find(span.begin(), span.end(), nib) == span.end()) {
+          for (size_t i = 0, n = span.size(); i < n; ++i) span.push_back(span[i] ^ nib);
+          order.push_back(x);
+        } else {
+          rest.push_back(x);
         }
-        if (indep) pick = x;
       }
-      if (K >= 5) {
-        if (pick < 0) pick = 4;
-        order.push_back(pick);
-        for (int x = 4; x < K; ++x)
-          if (x != pick) order.push_back(x);
-        for (int i = 0; i + 1 < K; ++i) d.store_bit[i] = (uint8_t)order[i];
-      }
+      order.insert(order.end(), rest.begin(), rest.end());
+      for (int i = 0; i + 1 < K; ++i) d.store_bit[i] = (uint8_t)order[i];
     }
     d.phase0 = (int)ps->phases.size();
-    d.nphases = 0;
     d.rop0 = (int)ps->rops.size();
-    // oriented: the tile bits and outer positions of first-colour spins
-    d.black_tile = 0;
-    d.black_outer = 0;
-    if (oriented) {
-      for (int q = 0; q < K; ++q)
-        if ((black >> d.tile_spin[q]) & 1ull) d.black_tile |= 1u << q;
-      for (int o = 0; o < M - K; ++o)
-        if ((black >> d.outer_spin[o]) & 1ull) d.black_outer |= 1ull << d.outer_pos[o];
-    }
-    std::vector<int> default_rb(RB);
-    for (int k = 0; k < RB; ++k) default_rb[k] = k;
-    std::vector<ROp> pending;  // element-wise ops waiting for the next phase
-    auto new_phase = [&](const std::vector<int> &rb) {
-      PhaseDesc ph;
-      memset(&ph, 0, sizeof ph);
-      uint32_t isreg = 0;
-      for (int k = 0; k < RB; ++k) ph.rb[k] = (uint8_t)rb[k], isreg |= 1u << rb[k];
-      // lane bits: nres non-register bits of distinct residues mod nres
-      // (bank-conflict free with the shared-memory swizzle), then the lowest left
-      std::vector<int> free_bits, lanes;
-      for (int b = 0; b < K; ++b)
-        if (!((isreg >> b) & 1)) free_bits.push_back(b);
-      uint32_t used = 0, res = 0;
-      for (int b : free_bits)
-        if ((int)lanes.size() < nres && !((res >> (b % nres)) & 1))
-          lanes.push_back(b), used |= 1u << b, res |= 1u << (b % nres);
-      for (int b : free_bits)
-        if (lanes.size() < 5 && !((used >> b) & 1)) lanes.push_back(b), used |= 1u << b;
-      for (int k = 0; k < 5; ++k) ph.lanes[k] = (uint8_t)lanes[k];
-      int nw = 0;
-      for (int b : free_bits)
-        if (!((used >> b) & 1)) ph.warps[nw++] = (uint8_t)b;
-      for (int k = 0; k < RB; ++k) ph.sm[k] = (uint16_t)slot_of(1u << ph.rb[k]);
-      for (int k = 0; k < 5; ++k) ph.tslot[k] = (uint16_t)slot_of(1u << ph.lanes[k]);
-      for (int k = 0; k < K - RB - 5; ++k) ph.tslot[5 + k] = (uint16_t)slot_of(1u << ph.warps[k]);
-      ph.op0 = (int)ps->rops.size();
-      ph.nops = 0;
-      for (const ROp &r : pending) ps->rops.push_back(r), ph.nops++;
-      pending.clear();
-      ps->phases.push_back(ph);
-      d.nphases++;
-    };
-    auto push_rop = [&](const ROp &r) {
-      ps->rops.push_back(r);
-      ps->phases.back().nops++;
-    };
-    bool last_is_diag = false;  // the last phase is a diagonal-only phase
-    // an element-wise op (the readout) between gates of one group: gates
-    // before it must all be applied first; it runs inside the phase that
-    // completes them (each thread reads its own amplitudes, whose gates so far
-    // acted within the thread's subcube)
-    int fence = -1;
-    ROp fence_op{};
-    auto flush = [&](std::vector<const Op *> &gates) {
-      if (gates.empty()) return true;
-      last_is_diag = false;
-      std::vector<std::pair<int, int>> pairs;
-      for (const Op *g : gates) pairs.push_back({g->u, g->v});
-      std::vector<uint32_t> sets;
-      std::vector<std::vector<int>> applied;
-      const int fz = fence < 0 ? (int)gates.size() : fence;
-      int pre_done = 0;
-      if (!plan_phases(K, pairs, RB, kPhaseBeam, fz, &sets, &applied, d.black_tile,
-                       oriented ? kOrientNbMask(RB) : 0u)) {
-        *err = "phase planning failed";
-        return false;
+    auto emit = [&](bool want_direct) {
+      d.nphases = 0;
+      ps->phases.resize(d.phase0);
+      ps->rops.resize(d.rop0);
+      // oriented: the tile bits and outer positions of first-colour spins
+      d.black_tile = 0;
+      d.black_outer = 0;
+      if (oriented) {
+        for (int q = 0; q < K; ++q)
+          if ((black >> d.tile_spin[q]) & 1ull) d.black_tile |= 1u << q;
+        for (int o = 0; o < M - K; ++o)
+          if ((black >> d.outer_spin[o]) & 1ull) d.black_outer |= 1ull << d.outer_pos[o];
       }
-      for (size_t k = 0; k < sets.size(); ++k) {
-        std::vector<int> rb;
-        if (oriented) {
-          // the NB first-colour bits first, then the others
-          for (int q = 0; q < K; ++q)
-            if (((sets[k] >> q) & 1) && ((d.black_tile >> q) & 1)) rb.push_back(q);
-          for (int q = 0; q < K; ++q)
-            if (((sets[k] >> q) & 1) && !((d.black_tile >> q) & 1)) rb.push_back(q);
-        } else {
-          for (int q = 0; q < K; ++q)
-            if ((sets[k] >> q) & 1) rb.push_back(q);
-          // register bit 0 is the pack bit of the complex64 kernel: the bit the
-          // fewest of this phase's gates touch (their arithmetic is scalar)
-          int pack = 0, best = 1 << 30;
-          for (int q = 0; q < (int)rb.size(); ++q) {
-            int n = 0;
-            for (int gi : applied[k]) n += (pairs[gi].first == rb[q]) + (pairs[gi].second == rb[q]);
-            if (n < best) best = n, pack = q;
-          }
-          std::rotate(rb.begin(), rb.begin() + pack, rb.begin() + pack + 1);
+      std::vector<int> default_rb(RB);
+      for (int k = 0; k < RB; ++k) default_rb[k] = k;
+      std::vector<ROp> pending;  // element-wise ops waiting for the next phase
+      d.direct = want_direct;
+      // lanes: bits that should be lane bits if they are not in registers
+      auto new_phase = [&](const std::vector<int> &rb, const std::vector<int> &prefer = {}) {
+        PhaseDesc ph;
+        memset(&ph, 0, sizeof ph);
+        uint32_t isreg = 0;
+        for (int k = 0; k < RB; ++k) ph.rb[k] = (uint8_t)rb[k], isreg |= 1u << rb[k];
+        // lane bits: nres non-register bits of distinct residues mod nres
+        // (bank-conflict free with the shared-memory swizzle), then the lowest left
+        std::vector<int> free_bits, lanes;
+        for (int b : prefer)
+          if (!((isreg >> b) & 1)) free_bits.push_back(b);
+        for (int b = 0; b < K; ++b)
+          if (!((isreg >> b) & 1) && std::find(free_bits.begin(), free_bits.end(), b) == free_bits.end())
+            free_bits.push_back(b);
+        uint32_t used = 0, res = 0;
+        for (int b : free_bits)
+          if ((int)lanes.size() < nres && !((res >> (b % nres)) & 1))
+            lanes.push_back(b), used |= 1u << b, res |= 1u << (b % nres);
+        for (int b : free_bits)
+          if (lanes.size() < 5 && !((used >> b) & 1)) lanes.push_back(b), used |= 1u << b;
+        for (int k = 0; k < 5; ++k) ph.lanes[k] = (uint8_t)lanes[k];
+        int nw = 0;
+        for (int b : free_bits)
+          if (!((used >> b) & 1)) ph.warps[nw++] = (uint8_t)b;
+        for (int k = 0; k < RB; ++k) ph.sm[k] = (uint16_t)slot_of(1u << ph.rb[k]);
+        for (int k = 0; k < 5; ++k) ph.tslot[k] = (uint16_t)slot_of(1u << ph.lanes[k]);
+        for (int k = 0; k < K - RB - 5; ++k) ph.tslot[5 + k] = (uint16_t)slot_of(1u << ph.warps[k]);
+        ph.op0 = (int)ps->rops.size();
+        ph.nops = 0;
+        for (const ROp &r : pending) ps->rops.push_back(r), ph.nops++;
+        pending.clear();
+        ps->phases.push_back(ph);
+        d.nphases++;
+      };
+      auto push_rop = [&](const ROp &r) {
+        ps->rops.push_back(r);
+        ps->phases.back().nops++;
+      };
+      bool last_is_diag = false;  // the last phase is a diagonal-only phase
+      // an element-wise op (the readout) between gates of one group: gates
+      // before it must all be applied first; it runs inside the phase that
+      // completes them (each thread reads its own amplitudes, whose gates so far
+      // acted within the thread's subcube)
+      int fence = -1;
+      ROp fence_op{};
+      auto flush = [&](std::vector<const Op *> &gates, bool at_end) {
+        if (gates.empty()) return true;
+        last_is_diag = false;
+        std::vector<std::pair<int, int>> pairs;
+        for (const Op *g : gates) pairs.push_back({g->u, g->v});
+        std::vector<uint32_t> sets;
+        std::vector<std::vector<int>> applied;
+        const int fz = fence < 0 ? (int)gates.size() : fence;
+        int pre_done = 0;
+        // a direct pass: its first phase holds tile bits 0 and 1, its last the
+        // ones written to them
+        const bool first_of = d.direct && d.nphases == 0, last_of = d.direct && at_end;
+        auto bit = [](int q) { return 1u << q; };
+        PhaseEnds ends;
+        if (first_of) ends.first = 3u, ends.avoid_first = 12u;
+        if (last_of) ends.last = bit(d.perm[0]) | bit(d.perm[1]), ends.avoid_last = bit(d.perm[2]) | bit(d.perm[3]);
+        if (!plan_phases(K, pairs, RB, kPhaseBeam, fz, &sets, &applied, d.black_tile,
+                         oriented ? kOrientNbMask(RB) : 0u, ends)) {
+          *err = "phase planning failed";
+          return false;
         }
-        new_phase(rb);
-        const int nbk = oriented ? __builtin_popcount(sets[k] & d.black_tile) : 0;
-        ps->phases.back().nb = (uint8_t)nbk;
-        for (int gi : applied[k]) {
-          const PlanGate g{gi, pairs[gi].first, pairs[gi].second};
-          int ku = (int)(std::find(rb.begin(), rb.end(), g.i) - rb.begin());
-          int kv = (int)(std::find(rb.begin(), rb.end(), g.j) - rb.begin());
-          if (ku > kv) std::swap(ku, kv);
-          int combo;
+        if (first_of && last_of && sets.size() == 1 && !(d.perm[0] == 0 && d.perm[1] == 1)) {
+          // one phase cannot hold both pairs as register bits 1 and 2
+          uint32_t s = ends.last;
+          for (uint32_t pool : {((1u << K) - 1u) & ~ends.avoid_last, (1u << K) - 1u})
+            for (int q = 0; q < K && __builtin_popcount(s) < RB; ++q)
+              if ((pool >> q) & 1u) s |= bit(q);
+          sets.push_back(s);
+          applied.push_back({});
+        }
+        for (size_t k = 0; k < sets.size(); ++k) {
+          std::vector<int> rb;
           if (oriented) {
-            // one bit of each colour: ku < nb <= kv
-            if (!(ku < nbk && kv >= nbk)) {
-              *err = "oriented phase: a gate joins two spins of one colour";
-              return false;
+            // the NB first-colour bits first, then the others
+            for (int q = 0; q < K; ++q)
+              if (((sets[k] >> q) & 1) && ((d.black_tile >> q) & 1)) rb.push_back(q);
+            for (int q = 0; q < K; ++q)
+              if (((sets[k] >> q) & 1) && !((d.black_tile >> q) & 1)) rb.push_back(q);
+          } else if (rounds) {
+            // the gates until the readout, then the ones after it
+            int split = -1;
+            std::vector<std::pair<int, int>> pg;
+            for (int gi : applied[k]) {
+              pg.push_back(pairs[gi]);
+              if (fence >= 0 && gi < fence && ++pre_done == fence) split = (int)pg.size();
             }
-            combo = 8 * ku + kv;
+            for (int q = 0; q < K; ++q)
+              if ((sets[k] >> q) & 1) rb.push_back(q);
+            std::vector<PhaseRound> rounds_of;
+            const bool first = first_of && k == 0, last = last_of && k + 1 == sets.size();
+            plan_rounds(pg, RB, split, last ? d.perm[0] : first ? 0 : -1, last ? d.perm[1] : first ? 1 : -1, &rb,
+                        &rounds_of);
+            if (last) new_phase(rb, {d.perm[2], d.perm[3]});
+            else new_phase(rb);
+            for (const PhaseRound &rd : rounds_of) {
+              if (rd.gates.empty()) {
+                push_rop(fence_op);
+                continue;
+              }
+              ROp r{};
+              r.kind = OP_ROUND;
+              r.arg = (uint8_t)rd.gates.size();
+              for (int i : rd.gates) r.coef |= 1 << rd.combo[i];
+              push_rop(r);
+              for (int i : rd.gates) {
+                ROp g{};
+                g.kind = OP_GATE;
+                g.combo = (uint8_t)rd.combo[i];
+                g.coef = gates[applied[k][i]]->coef;
+                push_rop(g);
+              }
+            }
+            continue;
           } else {
-            // combo = index of (ku, kv) among the RB(RB-1)/2 pairs, lexicographic
-            int base_idx = 0;
-            for (int i = 0; i < ku; ++i) base_idx += RB - 1 - i;
-            combo = base_idx + (kv - ku - 1);
+            for (int q = 0; q < K; ++q)
+              if ((sets[k] >> q) & 1) rb.push_back(q);
+            // register bit 0 is the pack bit of the complex64 kernel: the bit the
+            // fewest of this phase's gates touch (their arithmetic is scalar)
+            int pack = 0, best = 1 << 30;
+            for (int q = 0; q < (int)rb.size(); ++q) {
+              int n = 0;
+              for (int gi : applied[k]) n += (pairs[gi].first == rb[q]) + (pairs[gi].second == rb[q]);
+              if (n < best) best = n, pack = q;
+            }
+            std::rotate(rb.begin(), rb.begin() + pack, rb.begin() + pack + 1);
           }
-          ROp r{};
-          r.kind = OP_GATE;
-          r.combo = (uint8_t)combo;
-          r.coef = gates[g.bond]->coef;
+          new_phase(rb);
+          const int nbk = oriented ? __builtin_popcount(sets[k] & d.black_tile) : 0;
+          ps->phases.back().nb = (uint8_t)nbk;
+          for (int gi : applied[k]) {
+            const PlanGate g{gi, pairs[gi].first, pairs[gi].second};
+            int ku = (int)(std::find(rb.begin(), rb.end(), g.i) - rb.begin());
+            int kv = (int)(std::find(rb.begin(), rb.end(), g.j) - rb.begin());
+            if (ku > kv) std::swap(ku, kv);
+            int combo;
+            if (oriented) {
+              // one bit of each colour: ku < nb <= kv
+              if (!(ku < nbk && kv >= nbk)) {
+                *err = "oriented phase: a gate joins two spins of one colour";
+                return false;
+              }
+              combo = 8 * ku + kv;
+            } else {
+              // combo = index of (ku, kv) among the RB(RB-1)/2 pairs, lexicographic
+              int base_idx = 0;
+              for (int i = 0; i < ku; ++i) base_idx += RB - 1 - i;
+              combo = base_idx + (kv - ku - 1);
+            }
+            ROp r{};
+            r.kind = OP_GATE;
+            r.combo = (uint8_t)combo;
+            r.coef = gates[g.bond]->coef;
+            push_rop(r);
+            if (fence >= 0 && gi < fence && ++pre_done == fence) push_rop(fence_op);
+          }
+        }
+        fence = -1;
+        gates.clear();
+        return true;
+      };
+      std::vector<const Op *> gates;
+      for (int k = 0; k < d.nops; ++k) {
+        const Op &op = ps->ops[d.op0 + k];
+        if (op.kind == OP_GATE) {
+          gates.push_back(&op);
+          continue;
+        }
+        ROp r{};
+        r.kind = op.kind;
+        r.arg = op.arg;
+        if (op.kind == OP_REDUCE && !gates.empty() && fence < 0) {
+          fence = (int)gates.size();
+          fence_op = r;
+          continue;
+        }
+        if (!flush(gates, false)) return false;
+        if (op.kind == OP_DIAG) {
+          // the diagonal phase runs alone (its own phase, no register subcube)
+          if (!pending.empty()) new_phase(default_rb);
+          pending.push_back(r);
+          new_phase(default_rb);
+          last_is_diag = true;
+        } else if (d.nphases > 0 && pending.empty() && !last_is_diag) {
           push_rop(r);
-          if (fence >= 0 && gi < fence && ++pre_done == fence) push_rop(fence_op);
+        } else {
+          pending.push_back(r);
         }
       }
-      fence = -1;
-      gates.clear();
+      if (!flush(gates, true)) return false;
+      if (!pending.empty() || d.nphases == 0) new_phase(default_rb), d.direct = 0;
+      if (d.direct) {
+        const PhaseDesc &a = ps->phases[d.phase0], &b = ps->phases.back();
+        std::vector<int> out(K);  // output tile bit of each input tile bit
+        for (int q = 0; q < K; ++q) out[d.perm[q]] = q;
+        for (int i = 0; i < RB; ++i) d.in_reg[i] = d.tile_pos[a.rb[i]], d.out_reg[i] = d.tile_pos[out[b.rb[i]]];
+        for (int i = 0; i < K - RB; ++i) {
+          d.in_thr[i] = d.tile_pos[i < 5 ? a.lanes[i] : a.warps[i - 5]];
+          d.out_thr[i] = d.tile_pos[out[i < 5 ? b.lanes[i] : b.warps[i - 5]]];
+        }
+      }
+      d.nrops = (int)ps->rops.size() - d.rop0;
       return true;
     };
-    std::vector<const Op *> gates;
-    for (int k = 0; k < d.nops; ++k) {
-      const Op &op = ps->ops[d.op0 + k];
-      if (op.kind == OP_GATE) {
-        gates.push_back(&op);
-        continue;
-      }
-      ROp r{};
-      r.kind = op.kind;
-      r.arg = op.arg;
-      if (op.kind == OP_REDUCE && !gates.empty() && fence < 0) {
-        fence = (int)gates.size();
-        fence_op = r;
-        continue;
-      }
-      if (!flush(gates)) return false;
-      if (op.kind == OP_DIAG) {
-        // the diagonal phase runs alone (its own phase, no register subcube)
-        if (!pending.empty()) new_phase(default_rb);
-        pending.push_back(r);
-        new_phase(default_rb);
-        last_is_diag = true;
-      } else if (d.nphases > 0 && pending.empty() && !last_is_diag) {
-        push_rop(r);
-      } else {
-        pending.push_back(r);
+    // a direct pass (several tiles, gates first and last: a diagonal op there
+    // needs the tile in shared memory) where its two ends cost no phase more
+    const bool can = rounds && M > K && d.nops > 0 && ps->ops[d.op0].kind == OP_GATE &&
+                     ps->ops[d.op0 + d.nops - 1].kind != OP_DIAG;
+    if (!emit(false)) return false;
+    if (can) {
+      const PassDesc plain = d;
+      const std::vector<PhaseDesc> phases(ps->phases.begin() + d.phase0, ps->phases.end());
+      const std::vector<ROp> rops(ps->rops.begin() + d.rop0, ps->rops.end());
+      if (!emit(true)) return false;
+      if (!d.direct || d.nphases > plain.nphases) {
+        d = plain;
+        ps->phases.resize(d.phase0);
+        ps->phases.insert(ps->phases.end(), phases.begin(), phases.end());
+        ps->rops.resize(d.rop0);
+        ps->rops.insert(ps->rops.end(), rops.begin(), rops.end());
       }
     }
-    if (!flush(gates)) return false;
-    if (!pending.empty() || d.nphases == 0) new_phase(default_rb);
-    d.nrops = (int)ps->rops.size() - d.rop0;
+    // the diagonal op's tables (the same tile bits in every pass that has one)
+    if (d.diag >= 0) {
+      DiagTab t;
+      t.rb = (uint8_t)RB, t.L = (uint8_t)(K - RB);
+      t.words = (1 << RB) + (1 + RB) * (1 << (K - RB));
+      for (int i = 0; i < K; ++i) t.pos[i] = d.tile_pos[i];
+      if (ps->tab.words && memcmp(ps->tab.pos, t.pos, sizeof t.pos) != 0) {
+        *err = "diagonal ops on different tiles";
+        return false;
+      }
+      ps->tab = t;
+      for (int k = d.rop0; k < (int)ps->rops.size(); ++k)
+        if (ps->rops[k].kind == OP_DIAG) ps->rops[k].coef = ps->rops[k].arg * t.words;
+    }
     if (d.nphases > kMaxPassPhases || d.nrops > kMaxPassOps) {
       *err = "a sweep's register program exceeds the staging capacity";
       return false;
@@ -901,7 +1005,7 @@ static int plan_state_uncached(const spinrp_system &sys, int prec, Plan *plan, P
       if (ps->oriented) ps->black = sys.black;
     }
     ps->phased = ps->oriented || compile_phases(ps, sys.M, plan->K, ps->rb, prec, &err);
-    if (!ps->phased) ps->phases.clear(), ps->rops.clear();
+    if (!ps->phased) ps->phases.clear(), ps->rops.clear(), ps->tab = DiagTab{};
   }
   // every gate on two distinct bits of its tile; every store permutation a permutation
   for (const PassDesc &d : ps->desc) {
@@ -983,16 +1087,25 @@ static int set_smem_limits() {
   if (sizeof(R) == 4)
   {
     const cudaFuncAttribute a = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, false, false>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, false, false>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, true, false>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, true, false>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, false, true>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, false, true>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, true, true>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, true, true>, a, 8 << 14));
-    CUDA_TRY(cudaFuncSetAttribute(pipe_kernel<6, 13, false>, a, (int)kPipeSmem));
-    CUDA_TRY(cudaFuncSetAttribute(pipe_kernel<6, 13, true>, a, (int)kPipeSmem));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, false, false, false>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, true, false, false>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, false, false, false>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, true, false, false>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, false, false, true>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, false, false, true>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, true, false, true>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, true, false, true>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, false, true, false>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, false, true, false>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<5, true, true, false>, a, 8 << 14));
+    CUDA_TRY(cudaFuncSetAttribute(sweep2_kernel<6, true, true, false>, a, 8 << 14));
+#define PIPE_SMEM(V_)                                                               \
+  CUDA_TRY(cudaFuncSetAttribute(pipe_kernel<6, 13, false, V_>, a, (int)kPipeSmem)); \
+  CUDA_TRY(cudaFuncSetAttribute(pipe_kernel<6, 13, true, V_>, a, (int)kPipeSmem))
+    PIPE_SMEM(kPipeSparse);
+    PIPE_SMEM(kPipeDense);
+    PIPE_SMEM(kPipeDiag);
+#undef PIPE_SMEM
     CUDA_TRY(cudaFuncSetAttribute(resident_kernel<5, false>, a, (int)kResidentMaxSmem));
     CUDA_TRY(cudaFuncSetAttribute(resident_kernel<5, true>, a, (int)kResidentMaxSmem));
     CUDA_TRY(cudaFuncSetAttribute(resident_kernel<6, false>, a, (int)kResidentMaxSmem));
@@ -1016,13 +1129,13 @@ static unsigned sweep2_resident(int prec, int rb, int K, bool oriented) {
   const cudaError_t e =
       prec != SPINRP_C64
           ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2d_kernel, 1 << (K - 5), smem)
-      : rb == 6 ? (oriented ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<6, false, true>,
+      : rb == 6 ? (oriented ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<6, false, true, false>,
                                                                             1 << (K - 6), smem)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<6, false, false>,
+                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<6, false, false, true>,
                                                                             1 << (K - 6), smem))
-                : (oriented ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<5, false, true>,
+                : (oriented ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<5, false, true, false>,
                                                                             1 << (K - 5), smem)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<5, false, false>,
+                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<5, false, false, true>,
                                                                             1 << (K - 5), smem));
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -1041,7 +1154,7 @@ static unsigned pipe_grid(int prec, const Plan &plan, const PassSet &ps, int M, 
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pipe_kernel<6, 13, false>, kPipeThreads, kPipeSmem) !=
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pipe_kernel<6, 13, false, kPipeDiag>, kPipeThreads, kPipeSmem) !=
           cudaSuccess) {
     cudaGetLastError();
     return 0;
@@ -1147,6 +1260,7 @@ extern "C" int spinrp_state_create(const spinrp_system *sys, int prec, void *str
   hj.psites = st->psites;
   hj.site_series = st->site_series;
   hj.sops = (ROpRes *)(w + st->lay.sops);
+  hj.dtab = (uint64_t *)(w + st->lay.dtab);
   st->hjob = hj;
 
   auto up = [&](void *dst, const void *src, size_t n) -> cudaError_t {
@@ -1358,8 +1472,9 @@ extern "C" int spinrp_state_pipeline_timeout_check(spinrp_state *st, double *sec
   cudaEventRecord(e0, st->stream);
   // probe = 1: the producer issues no copies, so every wait of every block
   // runs out; nothing is written to the amplitudes or the series
-  pipe_kernel<6, 13, false><<<st->pipe_blocks, kPipeThreads, kPipeSmem, st->stream>>>(
-      st->d_job, 1, static_cast<float2 *>(st->psi), st->hjob.sops, 0, st->ps.desc[0], st->phases, st->M, err, 1);
+  pipe_kernel<6, 13, false, kPipeSparse><<<st->pipe_blocks, kPipeThreads, kPipeSmem, st->stream>>>(
+      st->d_job, 1, static_cast<float2 *>(st->psi), st->hjob.sops, st->hjob.qdiag, st->hjob.dtab, 0, st->ps.desc[0],
+      st->phases, st->M, err, 1);
   cudaEventRecord(e1, st->stream);
   ++g_launches;
   const cudaError_t le = cudaGetLastError();
@@ -1423,7 +1538,7 @@ static size_t resident_bytes(const Plan &plan, const PassSet &ps, int prec, bool
   if (ps.only < 0 || ps.first < 0 || ps.midstep < 0 || ps.last < 0) return 0;
   if (plan.M - ps.rb > 8) return 0;  // at most 256 threads per block
   const size_t b = (size_t(8) << plan.M) + sizeof(PhaseDesc) * ps.phases.size() +
-                   sizeof(ROpRes) * ps.rops.size();
+                   sizeof(ROpRes) * (ps.rops.size() + 1);  // a round reads one coefficient ahead
   return b <= kResidentMaxSmem ? b : 0;
 }
 
@@ -1481,32 +1596,42 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
     const int code = (c.rb == 6 ? 4 : 0) | (sites ? 2 : 0) | (c.oriented ? 1 : 0);
     const bool piped = c.pipe_blocks && K == 13 && code == 4;
     if (piped) {
-      if (c.njobs == 1)
-        pipe_kernel<6, 13, false><<<c.pipe_blocks, kPipeThreads, kPipeSmem, stream>>>(
-            c.jobs, 1, psi1, sops1, 0, pd, c.phases, c.M, c.pipe_err, 0);
-      else
-      {
-        pipe_kernel<6, 13, true><<<c.pipe_blocks, kPipeThreads, kPipeSmem, stream>>>(
-            c.jobs, c.njobs, static_cast<float2 *>(c.batch0.psi), c.batch0.sops, c.job_stride, pd, c.phases, c.M,
-            c.pipe_err, 0);
-        if (pd.has_reduce) {
-          CUDA_TRY(cudaGetLastError());
-          if (live) ++g_launches;
-          pipe_finalize_kernel<<<c.njobs, 128, 0, stream>>>(c.jobs, 1u << (c.M - 13), c.pipe_err);
-        }
+#define PIPE(B_, V_)                                                                                         \
+  pipe_kernel<6, 13, B_, V_><<<c.pipe_blocks, kPipeThreads, kPipeSmem, stream>>>(                            \
+      c.jobs, c.njobs, static_cast<float2 *>(j0.psi), j0.sops, j0.qdiag, j0.dtab, B_ ? c.job_stride : 0, pd, \
+      c.phases, c.M, c.pipe_err, 0)
+      const JobPtrs &j0 = c.njobs == 1 ? c.job0 : c.batch0;
+      const bool many = c.njobs > 1;
+      switch (2 * c.ps->variant(pass) + (many ? 1 : 0)) {
+        case 2 * kPipeSparse: PIPE(false, kPipeSparse); break;
+        case 2 * kPipeSparse + 1: PIPE(true, kPipeSparse); break;
+        case 2 * kPipeDense: PIPE(false, kPipeDense); break;
+        case 2 * kPipeDense + 1: PIPE(true, kPipeDense); break;
+        case 2 * kPipeDiag: PIPE(false, kPipeDiag); break;
+        default: PIPE(true, kPipeDiag); break;
+      }
+#undef PIPE
+      if (many && pd.has_reduce) {
+        CUDA_TRY(cudaGetLastError());
+        if (live) ++g_launches;
+        pipe_finalize_kernel<<<c.njobs, 128, 0, stream>>>(c.jobs, 1u << (c.M - 13), c.pipe_err);
       }
     } else {
-#define SW2(RB_, S_, O_) \
-  sweep2_kernel<RB_, S_, O_><<<grid, 1 << (K - RB_), sm2, stream>>>(c.jobs, psi1, sops1, pd, c.phases, c.M, ahead)
-      switch (code) {
-        case 0: SW2(5, false, false); break;
-        case 1: SW2(5, false, true); break;
-        case 2: SW2(5, true, false); break;
-        case 3: SW2(5, true, true); break;
-        case 4: SW2(6, false, false); break;
-        case 5: SW2(6, false, true); break;
-        case 6: SW2(6, true, false); break;
-        default: SW2(6, true, true); break;
+#define SW2(RB_, S_, O_, D_) \
+  sweep2_kernel<RB_, S_, O_, D_><<<grid, 1 << (K - RB_), sm2, stream>>>(c.jobs, psi1, sops1, pd, c.phases, c.M, ahead)
+      switch (code | (pd.direct ? 8 : 0)) {
+        case 0: SW2(5, false, false, false); break;
+        case 1: SW2(5, false, true, false); break;
+        case 2: SW2(5, true, false, false); break;
+        case 3: SW2(5, true, true, false); break;
+        case 4: SW2(6, false, false, false); break;
+        case 5: SW2(6, false, true, false); break;
+        case 6: SW2(6, true, false, false); break;
+        case 7: SW2(6, true, true, false); break;
+        case 8: SW2(5, false, false, true); break;
+        case 10: SW2(5, true, false, true); break;
+        case 12: SW2(6, false, false, true); break;
+        default: SW2(6, true, false, true); break;
       }
 #undef SW2
     }
@@ -1722,6 +1847,11 @@ extern "C" int spinrp_evolve(spinrp_state *st, double dt, int64_t steps, int ord
       ++g_launches;
       diag_kernel<<<(n + 127) / 128, 128, 0, st->stream>>>(st->d_job, layout_arg(st), st->M, dt);
       CUDA_TRY(cudaGetLastError());
+      if (st->ps.tab.words) {
+        ++g_launches;
+        diag_tab_kernel<<<(2 * st->ps.tab.words + 127) / 128, 128, 0, st->stream>>>(st->d_job, st->ps.tab, st->M);
+        CUDA_TRY(cudaGetLastError());
+      }
     }
     prof_mark(st, SPINRP_KERNEL_TABLES);
     st->coef_dt = dt;
@@ -2006,6 +2136,44 @@ std::string audit_sweep2(const PassDesc &d, const PhaseDesc *phases, int M, uint
         if (o != (s << 3) || ((o ^ ((uint32_t)ph.sm[0] << 3)) >> 3) >= T || (o >> 3) >= T) {
           snprintf(buf, sizeof buf, "phase %d pack walk out of place (g=%d)", p, g);
           return buf;
+        }
+      }
+    }
+  }
+  // a direct pass: every quad the first phase loads and the last stores, as the
+  // kernel walks them, four neighbouring amplitudes at a 32-byte boundary that
+  // are those of the phase's register index, each amplitude of the tile once
+  if (d.direct) {
+    if (d.nphases < 1) return "direct pass without phases";
+    auto quad_index = [&](int g) { return (gray(g) & 1) | ((gray(g) >> 1) << 3); };
+    for (int side = 0; side < 2; ++side) {
+      const PhaseDesc &ph = phases[d.phase0 + (side ? d.nphases - 1 : 0)];
+      const uint8_t *thr = side ? d.out_thr : d.in_thr, *reg = side ? d.out_reg : d.in_reg;
+      std::vector<char> hit(T, 0);
+      for (int tid = 0; tid < nt; ++tid) {
+        uint64_t off = base;
+        for (int k = 0; k < lognt; ++k) if ((tid >> k) & 1) off |= 1ull << thr[k];
+        uint32_t t0 = 0;
+        for (int k = 0; k < 5; ++k) t0 |= ((uint32_t)(tid >> k) & 1u) << ph.lanes[k];
+        for (int k = 0; k < lognt - 5; ++k) t0 |= ((uint32_t)(tid >> (5 + k)) & 1u) << ph.warps[k];
+        int64_t elem = (int64_t)off;
+        for (int g = 0; g < (1 << (rb - 2)); ++g) {
+          if (g) {
+            const int k = low_bit(g);
+            const int64_t dg = (int64_t)1 << reg[k ? k + 2 : 0];
+            elem += ((gray(g) >> k) & 1) ? dg : -dg;
+          }
+          if (elem < 0 || (elem & 3) || (uint64_t)elem + 3 >= N) return "direct quad out of range";
+          for (int q = 0; q < 4; ++q) {
+            const int i = quad_index(g) | q << 1;
+            uint32_t t = t0;
+            for (int k = 0; k < rb; ++k)
+              if ((i >> k) & 1) t |= 1u << ph.rb[k];
+            uint32_t to = 0;  // the tile bit order of the side
+            for (int x = 0; x < K; ++x)
+              to |= ((t >> (side ? d.perm[x] : x)) & 1u) << x;
+            if (t >= T || hit[t]++ || (uint64_t)elem + q != phys(to)) return "direct quad of other amplitudes";
+          }
         }
       }
     }
@@ -2332,11 +2500,23 @@ extern "C" int spinrp_system_plan_check(const spinrp_system *sys, int prec, doub
       int g = 0;
       for (int k = 0; k < ph.nops; ++k) {
         const ROp &r = ps.rops[ph.op0 + k];
-        if (r.kind == OP_GATE) {
+        if (r.kind == OP_ROUND) {
+          // its gates follow, in order and as its mask says
+          uint32_t m = 0;
+          bool ok = k + r.arg < ph.nops && r.arg > 0;
+          for (int i = 1; ok && i <= r.arg; ++i) {
+            const ROp &q = ps.rops[ph.op0 + k + i], &b4 = ps.rops[ph.op0 + k + i - 1];
+            ok = q.kind == OP_GATE && (i == 1 || q.combo > b4.combo);
+            m |= 1u << q.combo;
+          }
+          if (!ok || m != (uint32_t)r.coef) return fail(SPINRP_EINVAL, "plan_check: pass %zu phase %d: round", pi, p);
+        } else if (r.kind == OP_GATE) {
           check_rotate(B, ph.rb[KU[r.combo]], ph.rb[KV[r.combo]], r.coef);
           ++g;
         } else if (r.kind == OP_DIAG) {
           if (ph.nops != 1) return fail(SPINRP_EINVAL, "plan_check: diagonal op shares a phase");
+          if (d.diag < 0 || r.coef != r.arg * ps.tab.words || ps.tab.rb != ps.rb || ps.tab.L != K - ps.rb)
+            return fail(SPINRP_EINVAL, "plan_check: pass %zu: diagonal table", pi);
           check_diag(B, r.arg);
         } else {
           rb.push_back(check_reduce(B));
@@ -2590,6 +2770,7 @@ extern "C" int spinrp_batch_create(int njobs, const spinrp_system *const *system
     const size_t p_a = per; per = align256(per + sizeof(double) * M * M);
     const size_t p_q = per; per = align256(per + sizeof(uint64_t) * 2 * M * M);
     const size_t p_sops = per; per = align256(per + sizeof(ROpRes) * std::max<size_t>(g.ps.rops.size(), 1));
+    const size_t p_dtab = per; per = align256(per + sizeof(uint64_t) * 2 * g.ps.tab.words);
     const size_t total = o_job0 + per * n;
     cudaError_t e = cudaMalloc((void **)&g.dev, total);
     if (e != cudaSuccess) {
@@ -2621,6 +2802,7 @@ extern "C" int spinrp_batch_create(int njobs, const spinrp_system *const *system
       p.a = (double *)(j + p_a);
       p.qdiag = (uint64_t *)(j + p_q);
       p.sops = (ROpRes *)(j + p_sops);
+      p.dtab = (uint64_t *)(j + p_dtab);
       hs[k] = seeds[g.jobs[k]];
       for (int q = 0; q < g.nb; ++q) bv[q] = s.b[s.bonds[q].first * M + s.bonds[q].second];
       for (int q = 0; q < M * M; ++q) am[q] = s.a[q];
@@ -2933,6 +3115,11 @@ extern "C" int spinrp_batch_evolve(spinrp_batch *b, double dt, int64_t steps, in
         diag_kernel<<<dim3((2 * g.M * g.M + 127) / 128, n), 128, 0, b->stream>>>(g.d_jobs, group_layout(g),
                                                                                   g.M, dt);
         CUDA_TRY(cudaGetLastError());
+        if (g.ps.tab.words) {
+          ++g_launches;
+          diag_tab_kernel<<<dim3((2 * g.ps.tab.words + 127) / 128, n), 128, 0, b->stream>>>(g.d_jobs, g.ps.tab, g.M);
+          CUDA_TRY(cudaGetLastError());
+        }
       }
     }
     b->coef_dt = dt;

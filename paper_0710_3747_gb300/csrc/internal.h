@@ -16,6 +16,7 @@ enum OpKind : uint8_t {
   OP_GATE = 1,    // flip-flop gate on tile-local bits (u, v), coefficient index `coef`
   OP_DIAG = 2,    // e^{-i tau D} on every amplitude of the tile, tau variant `arg`
   OP_REDUCE = 3,  // accumulate N_up / N_dn of the readout spin into this pass's slot
+  OP_ROUND = 4,   // register-blocked plain complex64 programs: heads a round of gates (see ROp)
 };
 
 // One operation of a sweep, in tile-local bit indices.
@@ -48,6 +49,14 @@ struct PassDesc {
   int32_t rop0;         //   first op
   int32_t nrops;        //   and number of ops
   uint8_t store_bit[kMaxK];  // store: output tile bit (1..K-1) of each chunk-index bit
+  int32_t diag;         // S^zS^z variant of the pass's diagonal ops (0: dt/2, 1: dt), -1 without any
+  // a direct pass's first phase loads its subcubes from the state and its last
+  // phase stores them there (tile bits 0 and 1, in the output order for the
+  // store, are register bits 1 and 2); physical positions of the thread-index
+  // and register bits of those two phases
+  int32_t direct;
+  uint8_t in_thr[kMaxK - 5], out_thr[kMaxK - 5];
+  uint8_t in_reg[6], out_reg[6];
   // oriented states (see Orientation below): tile bits and outer physical
   // positions that hold spins of the first colour, input layout
   uint32_t black_tile;
@@ -98,7 +107,12 @@ inline uint32_t swizzle_slot16(uint32_t t) { return t ^ (((t >> 3) ^ (t >> 6) ^ 
 
 // Op of a phase: GATE acts on register bits given by `combo` (index of the
 // pair (ku < kv) among the RB(RB-1)/2 pairs, lexicographic; in an oriented
-// program ku < nb <= kv and combo = 8 ku + kv); DIAG / REDUCE as in Op.
+// program ku < nb <= kv and combo = 8 ku + kv); DIAG / REDUCE as in Op (a
+// DIAG keeps its table's offset in `coef`).
+// Plain complex64 programs group a phase's gates into rounds.  A round's gates
+// (`arg` of them) follow its ROUND op in ascending order of their combos and
+// `coef` has the bit of each: the kernel walks the pairs in order once, testing
+// bits, instead of jumping to each gate's code.
 struct ROp {
   uint8_t kind;
   uint8_t combo;
@@ -109,12 +123,26 @@ struct ROp {
 
 struct GateCoef;
 
+// Tables of the diagonal op of a register-blocked plan.  With tile bits 0..L-1
+// taken from the thread index and the RB high ones walked by every thread,
+// Theta(x) = sum_{p<p'} q_pp' sigma sigma' is a part of the high bits, a part
+// of the thread's bits, the thread bits' fields on the high bits and the outer
+// spins' fields; only the last depend on the tile.  The others are laid out
+// once per dt as 64-bit turns: per variant (dt/2, dt) `words` words, 2^rb high
+// parts, 2^L thread parts and rb x 2^L fields.  (Every pass with a diagonal op
+// spans the first segment's tile in the step-boundary layout.)
+struct DiagTab {
+  int32_t words = 0;      // 0: the plan has no diagonal op
+  uint8_t rb = 0, L = 0;
+  uint8_t pos[kMaxK] = {};  // physical position of each tile bit
+};
+
 // A phase op with its FP32 gate coefficients resolved for the current dt (one
 // array per job, rebuilt with the gate table), 16 bytes for 16-byte copies.
 struct ROpRes {
   uint8_t kind, combo, arg, pad;
   float t, s;  // shear coefficients tan(theta/2), sin(theta) of a gate
-  uint32_t pad2;
+  uint32_t tab;  // diagonal op: offset of its variant's table (8-byte words)
 };
 static_assert(sizeof(ROpRes) == 16, "ROpRes is copied in 16-byte pieces");
 static_assert(sizeof(PhaseDesc) % 4 == 0, "PhaseDesc is copied in 4-byte pieces");
@@ -135,6 +163,7 @@ struct JobPtrs {
                            // norm, column 1 + q the weight with spin q up (q logical, 0-based);
                            // nullptr when only spin 1 is read out
   double *site_series;     // all-site readout: P of spin q at entry k in site_series[k * M + q]
+  uint64_t *dtab;          // tables of the diagonal op (DiagTab)
   ROpRes *sops;            // register-blocked program ops with resolved coefficients
 };
 
@@ -173,6 +202,14 @@ int report_error(int code, const char *msg);
 bool build_plan(int M, const std::vector<std::pair<int, int>> &bonds, int K, int c, Plan *plan,
                 std::string *err);
 
+// Constraints of a direct pass on its phases: tile bits that the first set and
+// the last set hold, and ones that they rather leave to the thread index (the
+// next bits of the address, so that a warp's accesses fill 128-byte lines).
+// A last set may come without gates.
+struct PhaseEnds {
+  uint32_t first = 0, last = 0, avoid_first = 0, avoid_last = 0;
+};
+
 // Phases of a pass for the register-blocked kernel: gates (pairs of tile bits,
 // in order) cut into register sets of RB of the K tile bits; sets[k] (bit
 // mask) applies the gates applied[k], in an order that keeps every bit's gate
@@ -183,6 +220,19 @@ bool build_plan(int M, const std::vector<std::pair<int, int>> &bonds, int K, int
 // oriented kernel's colour patterns).  False if a gate cannot be placed.
 bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, int beam, int fence,
                  std::vector<uint32_t> *sets, std::vector<std::vector<int>> *applied,
-                 uint32_t black = 0, uint32_t nb_allowed = 0);
+                 uint32_t black = 0, uint32_t nb_allowed = 0, const PhaseEnds &ends = PhaseEnds());
+
+// Rounds of one phase's gates (pairs of tile bits, in order): chooses the order
+// of the RB register bits in *rb (bit 0 is the pack bit, whose gates are
+// scalar) and cuts the gates into rounds, walks over the register-bit pairs in
+// lexicographic order that keep every bit's gate sequence, for few rounds and few gates on the pack bit.  An empty round
+// stands for the readout after the first `split` gates (split < 0: none).
+// fix1, fix2: tile bits that register bits 1 and 2 hold (-1: any).
+struct PhaseRound {
+  std::vector<int> gates;  // indices into the phase's gates, in execution order
+  std::vector<int> combo;  // register-bit pair of every gate of the phase
+};
+void plan_rounds(const std::vector<std::pair<int, int>> &gates, int RB, int split, int fix1, int fix2,
+                 std::vector<int> *rb, std::vector<PhaseRound> *rounds);
 
 }  // namespace spinrp

@@ -408,7 +408,8 @@ __global__ void resolve_ops_kernel(const JobPtrs *__restrict__ jobs, const ROp *
   const JobPtrs &jp = jobs[blockIdx.y];
   const ROp r = rops[i];
   ROpRes o;
-  o.kind = r.kind, o.combo = r.combo, o.arg = r.arg, o.pad = 0, o.pad2 = 0;
+  o.kind = r.kind, o.combo = r.combo, o.arg = r.arg, o.pad = 0;
+  o.tab = r.kind == OP_GATE ? 0u : (uint32_t)r.coef;  // a diagonal op's table, a round's gates
   o.t = 0.f, o.s = 0.f;
   if (r.kind == OP_GATE) {
     const GateCoef g = jp.coefs[r.coef];
@@ -436,6 +437,39 @@ __global__ void diag_kernel(const JobPtrs *__restrict__ jobs, LayoutArg lay, int
     val = ((uint64_t)llrint(f * 9.223372036854775808e18)) << 1;
   }
   q[k] = val;
+}
+
+// A job's diagonal tables (see DiagTab), from the pair phases of diag_kernel:
+// one thread per entry, the sums exact modulo 2^64.
+__global__ void diag_tab_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ DiagTab t, int M) {
+  const JobPtrs &jp = jobs[blockIdx.y];
+  const int nr = 1 << t.rb, nt = 1 << t.L;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x, v = e >= t.words, i = e - v * t.words;
+  if (e >= 2 * t.words) return;
+  const uint64_t *__restrict__ q = jp.qdiag + (size_t)v * M * M;
+  // the pair phases among n tile bits from bit b0, signs from the bits of x
+  auto pairs = [&](int b0, int n, int x) {
+    uint64_t s = 0;
+    for (int a = 0; a < n; ++a)
+      for (int b = a + 1; b < n; ++b) {
+        const uint64_t y = q[t.pos[b0 + a] * M + t.pos[b0 + b]];
+        s += (((x >> a) ^ (x >> b)) & 1) ? (0ull - y) : y;
+      }
+    return s;
+  };
+  uint64_t r = 0;
+  if (i < nr) {
+    r = pairs(t.L, t.rb, i);
+  } else if (i < nr + nt) {
+    r = pairs(0, t.L, i - nr);
+  } else {
+    const int k = ((i - nr) >> t.L) - 1, x = (i - nr) & (nt - 1);
+    for (int b = 0; b < t.L; ++b) {
+      const uint64_t y = q[t.pos[t.L + k] * M + t.pos[b]];
+      r += ((x >> b) & 1) ? y : (0ull - y);
+    }
+  }
+  jp.dtab[e] = r;
 }
 
 // ---------------------------------------------------------------------------
@@ -780,40 +814,65 @@ __device__ __forceinline__ void gate_packbit(u64 (&RE)[NP], u64 (&IM)[NP], float
   }
 }
 
-// combo = index of (ku < kv) among the RB(RB-1)/2 register-bit pairs in
-// lexicographic order: the first RB-1 pair the pack bit (ku = 0).
-__device__ __forceinline__ void gate_combo(u64 (&RE)[16], u64 (&IM)[16], int combo, float t, float s) {
-  switch (combo) {
-    case 0: gate_packbit<16, 0>(RE, IM, t, s); break;
-    case 1: gate_packbit<16, 1>(RE, IM, t, s); break;
-    case 2: gate_packbit<16, 2>(RE, IM, t, s); break;
-    case 3: gate_packbit<16, 3>(RE, IM, t, s); break;
-    case 4: gate_packed<16, 0, 1>(RE, IM, t, s); break;
-    case 5: gate_packed<16, 0, 2>(RE, IM, t, s); break;
-    case 6: gate_packed<16, 0, 3>(RE, IM, t, s); break;
-    case 7: gate_packed<16, 1, 2>(RE, IM, t, s); break;
-    case 8: gate_packed<16, 1, 3>(RE, IM, t, s); break;
-    default: gate_packed<16, 2, 3>(RE, IM, t, s); break;
+// Gate on the register bits (ku, kv) of combo C = index of the pair ku < kv in
+// lexicographic order; the first RB - 1 pairs have the pack bit (ku = 0).
+template <int NP, int C>
+__device__ __forceinline__ void gate_of(u64 (&RE)[NP], u64 (&IM)[NP], float t, float s) {
+  constexpr int RB = NP == 16 ? 5 : 6;
+  static_assert(NP == 1 << (RB - 1), "five or six register bits");
+  if constexpr (C < RB - 1) {
+    gate_packbit<NP, C>(RE, IM, t, s);
+  } else {
+    constexpr int D = C - (RB - 1);  // among the pairs of bits 1..RB-1
+    constexpr int U = D < RB - 2 ? 0 : D < 2 * RB - 5 ? 1 : D < 3 * RB - 9 ? 2 : 3;
+    constexpr int V = D - (U * (2 * (RB - 1) - U - 1)) / 2 + U + 1;
+    static_assert(U < V && V < RB - 1, "a pair of register bits");
+    gate_packed<NP, U, V>(RE, IM, t, s);
   }
 }
+
+// The gate of a pair by a jump (sparse passes of the pipelined sweep).
 __device__ __forceinline__ void gate_combo(u64 (&RE)[32], u64 (&IM)[32], int combo, float t, float s) {
   switch (combo) {
-    case 0: gate_packbit<32, 0>(RE, IM, t, s); break;
-    case 1: gate_packbit<32, 1>(RE, IM, t, s); break;
-    case 2: gate_packbit<32, 2>(RE, IM, t, s); break;
-    case 3: gate_packbit<32, 3>(RE, IM, t, s); break;
-    case 4: gate_packbit<32, 4>(RE, IM, t, s); break;
-    case 5: gate_packed<32, 0, 1>(RE, IM, t, s); break;
-    case 6: gate_packed<32, 0, 2>(RE, IM, t, s); break;
-    case 7: gate_packed<32, 0, 3>(RE, IM, t, s); break;
-    case 8: gate_packed<32, 0, 4>(RE, IM, t, s); break;
-    case 9: gate_packed<32, 1, 2>(RE, IM, t, s); break;
-    case 10: gate_packed<32, 1, 3>(RE, IM, t, s); break;
-    case 11: gate_packed<32, 1, 4>(RE, IM, t, s); break;
-    case 12: gate_packed<32, 2, 3>(RE, IM, t, s); break;
-    case 13: gate_packed<32, 2, 4>(RE, IM, t, s); break;
-    default: gate_packed<32, 3, 4>(RE, IM, t, s); break;
+    case 0: gate_of<32, 0>(RE, IM, t, s); break;
+    case 1: gate_of<32, 1>(RE, IM, t, s); break;
+    case 2: gate_of<32, 2>(RE, IM, t, s); break;
+    case 3: gate_of<32, 3>(RE, IM, t, s); break;
+    case 4: gate_of<32, 4>(RE, IM, t, s); break;
+    case 5: gate_of<32, 5>(RE, IM, t, s); break;
+    case 6: gate_of<32, 6>(RE, IM, t, s); break;
+    case 7: gate_of<32, 7>(RE, IM, t, s); break;
+    case 8: gate_of<32, 8>(RE, IM, t, s); break;
+    case 9: gate_of<32, 9>(RE, IM, t, s); break;
+    case 10: gate_of<32, 10>(RE, IM, t, s); break;
+    case 11: gate_of<32, 11>(RE, IM, t, s); break;
+    case 12: gate_of<32, 12>(RE, IM, t, s); break;
+    case 13: gate_of<32, 13>(RE, IM, t, s); break;
+    default: gate_of<32, 14>(RE, IM, t, s); break;
   }
+}
+__device__ __forceinline__ void gate_combo(u64 (&)[16], u64 (&)[16], int, float, float) {}  // walks only
+
+// One round of a phase's gates: the pairs of `mask` in ascending order of C,
+// coefficients from consecutive ops.  Straight code with a test before each
+// pair: gates that run follow each other in the instruction stream, and the
+// next gate's coefficients load while this one computes.  A jump per gate (a
+// switch on the pair) took about 280 cycles a gate for a lone warp, most of it
+// the jump and the instruction fetch after it; this takes about 57 (a six-gate
+// phase of a 2^12 tile 2850 -> 1890 cycles).  One walk direction only: with a second, descending copy the sweep's code outgrew the
+// instruction cache (stalls on instructions 1.7 per issue against 0.3, 15 %
+// slower on ladders); the phase planner orders the register bits so that one
+// ascending walk takes nearly every phase.
+template <int NP, int C = 0>
+__device__ __forceinline__ void run_round(u64 (&RE)[NP], u64 (&IM)[NP], uint32_t mask, const ROpRes *op, float2 ts) {
+  constexpr int RB = NP == 16 ? 5 : 6, NC = RB * (RB - 1) / 2;
+  if ((mask >> C) & 1u) {
+    const float2 now = ts;
+    ++op;
+    ts = make_float2(op->t, op->s);
+    gate_of<NP, C>(RE, IM, now.x, now.y);
+  }
+  if constexpr (C + 1 < NC) run_round<NP, C + 1>(RE, IM, mask, op, ts);
 }
 
 // lowest set bit of a compile-time g in 1..31 (Gray-code walk)
@@ -925,121 +984,141 @@ __device__ __forceinline__ uint32_t thread_origin(const PhaseDesc &ph, int tid, 
   return t0;
 }
 
-// The diagonal phase e^{-i tau D}, amplitude by amplitude in shared memory.
+// Fields of the outer spins on a tile's bits, sH[t] = sum_o sigma_o q_to, and
+// their own part of Theta, sH[K] (exact modulo 2^64), by the 2^lognt threads
+// tid of the group: eight lanes share each entry, so the loads of a row are in
+// flight together.  The group's next barrier publishes them.
+__device__ __forceinline__ void diag_fields(const PassDesc &d, uint64_t base, int tid, int lognt, int M,
+                                            const uint64_t *__restrict__ qdiag, uint64_t *sH) {
+  const int K = d.K, nout = M - K, part = tid & 7;
+  const uint64_t *__restrict__ q = qdiag + (size_t)d.diag * M * M;
+  for (int t0 = 0; t0 <= K; t0 += 1 << (lognt - 3)) {
+    const int t = t0 + (tid >> 3);
+    uint64_t v = 0;
+    if (t < K) {
+      const int row = d.tile_pos[t] * M;
+      for (int o = part; o < nout; o += 8) {
+        const int po = d.outer_pos[o];
+        const uint64_t x = q[row + po];
+        v += ((base >> po) & 1ull) ? x : (0ull - x);
+      }
+    } else if (t == K) {
+      for (int o = part; o < nout; o += 8) {
+        const int pa = d.outer_pos[o];
+        uint64_t r = 0;
+        for (int o2 = o + 1; o2 < nout; ++o2) {
+          const int pb = d.outer_pos[o2];
+          const uint64_t x = q[pa * M + pb];
+          r += ((base >> pb) & 1ull) ? x : (0ull - x);
+        }
+        v += ((base >> pa) & 1ull) ? r : (0ull - r);
+      }
+    }
+#pragma unroll
+    for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (part == 0 && t <= K) sH[t] = v;
+  }
+}
+
+// e^{i theta} of two angles given as turns x 2^32 plus an eighth of a turn:
+// (re, im) packed.  The top two bits are the quarter turn, the others minus the
+// eighth the remainder y x pi/4, |y| <= 1, whose sine and cosine are minimax
+// polynomials in y^2 (Remez exchange; pi/4 split in two floats, the cosine's
+// leading coefficient rounded before the others were fitted, so that neither
+// the angle's scale nor the modulus is biased).  Errors against 64 bits over
+// all remainders: rms 1.44e-8 (sine) and 1.87e-8 (cosine), where correctly
+// rounded values have 1.42e-8 and 1.81e-8.
+__device__ __forceinline__ void cis_eighths(uint32_t a0, uint32_t a1, u64 &re, u64 &im) {
+  const float f0 = (float)((int)(a0 & 0x3fffffffu) - 0x20000000);
+  const float f1 = (float)((int)(a1 & 0x3fffffffu) - 0x20000000);
+  const float k = 1.862645149230957e-09f;  // 2^-29
+  const u64 y = mul2(pack2(f0, f1), pack2(k, k)), z = mul2(y, y);
+  auto c2 = [](float v) { return pack2(v, v); };
+  u64 p = fma2(c2(-3.58774269e-05f), z, c2(0.00248987228f));
+  p = fma2(p, z, c2(-0.0807453692f));
+  p = fma2(p, z, c2(-3.26817364e-08f));
+  const float2 s = unpack2(fma2(y, c2(0.785398185f), mul2(p, y)));
+  u64 q = fma2(c2(3.50271148e-06f), z, c2(-0.000325882982f));
+  q = fma2(q, z, c2(0.0158542898f));
+  q = fma2(q, z, c2(-0.308425128f));
+  const float2 c = unpack2(fma2(q, z, c2(1.0f)));
+  // quarter turns 0..3: (c, s), (-s, c), (-c, -s), (s, -c)
+  const bool w0 = (a0 & 0x40000000u) != 0, w1 = (a1 & 0x40000000u) != 0;
+  const uint32_t r0 = __float_as_uint(w0 ? s.x : c.x) ^ ((a0 ^ (a0 << 1)) & 0x80000000u);
+  const uint32_t r1 = __float_as_uint(w1 ? s.y : c.y) ^ ((a1 ^ (a1 << 1)) & 0x80000000u);
+  const uint32_t i0 = __float_as_uint(w0 ? c.x : s.x) ^ (a0 & 0x80000000u);
+  const uint32_t i1 = __float_as_uint(w1 ? c.y : s.y) ^ (a1 & 0x80000000u);
+  re = pack2(__uint_as_float(r0), __uint_as_float(r1));
+  im = pack2(__uint_as_float(i0), __uint_as_float(i1));
+}
+
+// The diagonal op e^{-i tau D} on a tile in shared memory, by the 2^lognt
+// threads tid of the group: thread tid takes the amplitudes t = tid + 2^lognt e,
+// e = 0..2^RB - 1.  Theta(t) is the table's thread part, plus the fields on the
+// thread's bits, plus sum_k sigma_k g_k + (register part e) over the RB high
+// tile bits, g_k the field of the thread's bits and of the outer spins on bit
+// k: two 64-bit additions an amplitude (exact), the register part one
+// broadcast load for two.  A loop over eight amplitudes at a time, out of
+// line: bound by latency and, when unrolled over all 2^RB, by instruction
+// fetch (its code runs once a tile and no longer fits the instruction cache
+// next to the gates; applied inside a phase's registers it also spilled, 0.73
+// of the speed on ladders that never run it).  One tile of 2^12, a warp per
+// scheduler: about 10^4 cycles untabulated and unrolled, 4300 so.
 // ORIENT: amplitudes of odd orientation are stored (Im, Re) and take the
 // conjugate phase (the stored word is i conj(psi), and i conj(psi e^{ia}) =
-// i conj(psi) e^{-ia}).  Kept out of line: only systems with S^zS^z terms run
-// it, and the sweep's gate code stays smaller (measured 2 % faster on
-// dipolar stars, unchanged on XY ladders).
-template <int RB, bool ORIENT, typename Sync>
-__device__ __noinline__ void diag_phase(float2 *tile2, const PassDesc &d, const PhaseDesc &ph,
-                                           const ROpRes &op, uint64_t base, int tid, int lognt, int M,
-                                           const uint64_t *__restrict__ qdiag, uint64_t *sH, uint64_t *sQ,
-                                           uint64_t *sOut, uint32_t s0, const uint32_t (&sm)[RB], Sync sync) {
-  constexpr int NA = 1 << RB;
-  const int K = d.K, nt = 1 << lognt;
-  const int nout = M - K;
-  // Theta(x) = sum_{p<p'} q_pp' sigma_p sigma_p' (mod 2^64) split into
-  // outer-outer (sOut), outer-tile (sH) and tile-tile (sQ) parts
-  uint32_t t0 = 0;
-  for (int k = 0; k < 5; ++k) t0 |= ((uint32_t)(tid >> k) & 1u) << ph.lanes[k];
-  for (int k = 0; k < lognt - 5; ++k) t0 |= ((uint32_t)(tid >> (5 + k)) & 1u) << ph.warps[k];
-  const uint64_t *q = qdiag + (size_t)op.arg * M * M;
-  if (tid < K) {
-    const int pp = d.tile_pos[tid];
-    uint64_t h = 0;
-    for (int o = 0; o < nout; ++o) {
-      const int po = d.outer_pos[o];
-      const uint64_t v = q[pp * M + po];
-      h += ((base >> po) & 1ull) ? v : (0ull - v);
+// i conj(psi) e^{-ia}).
+template <int RB, bool ORIENT>
+__device__ __noinline__ void diag_tile(float2 *tile2, const uint64_t *__restrict__ tab, const uint64_t *sH, int K,
+                                       int tid, int lognt, uint32_t black, uint32_t outer_par) {
+  const uint64_t *__restrict__ tthr = tab + (1 << RB) + tid;
+  uint64_t g[RB], base = sH[K] + tthr[0] + (1ull << 61);
+#pragma unroll
+  for (int k = 0; k < RB; ++k) g[k] = sH[lognt + k] + tthr[(size_t)(k + 1) << lognt];
+#pragma unroll
+  for (int b = 0; b < kMaxK - 5; ++b)
+    if (b < lognt) {
+      const uint64_t h = sH[b];
+      base += ((tid >> b) & 1) ? h : (0ull - h);
     }
-    sH[tid] = h;
-  } else if (tid == K) {
-    uint64_t s = 0;
-    for (int o = 0; o < nout; ++o)
-      for (int o2 = o + 1; o2 < nout; ++o2) {
-        const int pa = d.outer_pos[o], pb = d.outer_pos[o2];
-        const uint64_t v = q[pa * M + pb];
-        s += (((base >> pa) ^ (base >> pb)) & 1ull) ? (0ull - v) : v;
+  uint32_t ds[RB];
+#pragma unroll
+  for (int k = 0; k < RB; ++k) base -= g[k], g[k] += g[k], ds[k] = slot(1u << (lognt + k)) << 3;
+  char *const tb = reinterpret_cast<char *>(tile2);
+  const uint32_t o0 = slot((uint32_t)tid) << 3;
+#pragma unroll 1
+  for (int hi = 0; hi < (1 << (RB - 3)); ++hi) {
+    uint64_t lin = base;
+    uint32_t o = o0;
+#pragma unroll
+    for (int k = 3; k < RB; ++k)
+      if ((hi >> (k - 3)) & 1) lin += g[k], o ^= ds[k];
+    const ulonglong2 *__restrict__ treg = reinterpret_cast<const ulonglong2 *>(tab) + 4 * hi;
+    float2 v[8];
+    uint32_t oe[8];
+    u64 c[4], sn[4];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      oe[e] = o ^ ((e & 1) ? ds[0] : 0) ^ ((e & 2) ? ds[1] : 0) ^ ((e & 4) ? ds[2] : 0);
+      v[e] = *reinterpret_cast<const float2 *>(tb + oe[e]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {  // amplitudes e = 8 hi + 2 i and the next one
+      const uint64_t l = lin + ((i & 1) ? g[1] : 0) + ((i & 2) ? g[2] : 0);
+      const ulonglong2 t = treg[i];
+      cis_eighths((uint32_t)((l + t.x) >> 32), (uint32_t)((l + g[0] + t.y) >> 32), c[i], sn[i]);
+      if constexpr (ORIENT) {
+        const uint32_t e = 8u * hi + 2u * i, ta = (uint32_t)tid | (e << lognt);
+        const uint32_t pa = (__popc(ta & black) ^ outer_par) & 1u, pb = pa ^ ((black >> lognt) & 1u);
+        sn[i] ^= ((u64)pa << 31) | ((u64)pb << 63);
       }
-    *sOut = s;
-  }
-  for (int w = tid; w < K * K; w += nt) sQ[w] = q[d.tile_pos[w / K] * M + d.tile_pos[w % K]];
-  sync();
-  uint32_t isreg = 0;
-  for (int k = 0; k < RB; ++k) isreg |= 1u << ph.rb[k];
-  // fixed part (tile bits from the thread index) once per thread
-  uint64_t th0 = *sOut;
-  for (int x = 0; x < K; ++x) {
-    if ((isreg >> x) & 1u) continue;
-    const uint32_t bx = (t0 >> x) & 1u;
-    th0 += bx ? sH[x] : (0ull - sH[x]);
-    for (int y = x + 1; y < K; ++y) {
-      if ((isreg >> y) & 1u) continue;
-      th0 += (bx ^ ((t0 >> y) & 1u)) ? (0ull - sQ[x * K + y]) : sQ[x * K + y];
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 cc = unpack2(c[i]), ss = unpack2(sn[i]);
+      *reinterpret_cast<float2 *>(tb + oe[2 * i]) = cmul(v[2 * i], make_float2(cc.x, ss.x));
+      *reinterpret_cast<float2 *>(tb + oe[2 * i + 1]) = cmul(v[2 * i + 1], make_float2(cc.y, ss.y));
     }
   }
-  // field on each register bit from the fixed bits, once per thread
-  uint64_t G[RB];
-#pragma unroll
-  for (int k = 0; k < RB; ++k) {
-    const int rk = ph.rb[k];
-    uint64_t g = sH[rk];
-    for (int x = 0; x < K; ++x) {
-      if ((isreg >> x) & 1u) continue;
-      g += ((t0 >> x) & 1u) ? sQ[x * K + rk] : (0ull - sQ[x * K + rk]);
-    }
-    G[k] = g;
-  }
-  // the register combinations in Gray-code order: with sigma_k = +1 for a
-  // set bit and -1 for a clear one, Theta = th0 + sum_k sigma_k G_k +
-  // sum_{k<l} sigma_k sigma_l Q_kl; flipping bit k changes Theta by
-  // -2 sigma_k F_k, F_k = G_k + sum_{l!=k} sigma_l Q_kl its field, and
-  // every other field F_l by -2 sigma_k Q_kl (exact, modulo 2^64)
-  uint64_t Qr[RB][RB], F[RB];
-#pragma unroll
-  for (int k = 0; k < RB; ++k)
-#pragma unroll
-    for (int l = 0; l < RB; ++l)
-      Qr[k][l] = k == l ? 0ull : sQ[ph.rb[k < l ? k : l] * K + ph.rb[k < l ? l : k]];
-  uint64_t th = th0;
-#pragma unroll
-  for (int k = 0; k < RB; ++k) {
-    th -= G[k];
-    F[k] = G[k];
-#pragma unroll
-    for (int l = 0; l < RB; ++l) {
-      if (l == k) continue;
-      F[k] -= Qr[k][l];
-      if (l > k) th += Qr[k][l];
-    }
-  }
-  uint32_t s = s0;
-  // orientation of the current amplitude and of each register bit
-  uint32_t ori = 0, obit[RB];
-  if constexpr (ORIENT) {
-    ori = (__popc(t0 & d.black_tile) ^ __popcll(base & d.black_outer)) & 1u;
-#pragma unroll
-    for (int k = 0; k < RB; ++k) obit[k] = (d.black_tile >> ph.rb[k]) & 1u;
-  }
-#pragma unroll
-  for (int g = 0; g < NA; ++g) {
-    if (g) {
-      const int k = ctz6(g);
-      // sigma_k before the flip: +1 when the bit is set in gray(g - 1)
-      const bool was_up = ((((g - 1) ^ ((g - 1) >> 1)) >> k) & 1) != 0;
-      th += was_up ? (0ull - 2ull * F[k]) : 2ull * F[k];
-#pragma unroll
-      for (int l = 0; l < RB; ++l)
-        if (l != k) F[l] += was_up ? (0ull - 2ull * Qr[l][k]) : 2ull * Qr[l][k];
-      s ^= sm[k];
-      if constexpr (ORIENT) ori ^= obit[k];
-    }
-    float2 e = cis_turns(th, 0.0f);
-    if constexpr (ORIENT) e.y = ori ? -e.y : e.y;
-    tile2[s] = cmul(tile2[s], e);
-  }
-  sync();
 }
 
 // Register-blocked phases of an oriented program (see Orientation): the
@@ -1219,17 +1298,91 @@ __device__ __forceinline__ void oriented_phase(float2 *tile2, const PassDesc &d,
   }
 }
 
+// A thread's first-phase subcube straight from the state (direct passes): tile
+// bits 0 and 1 are register bits 1 and 2, so each 32-byte load brings four
+// neighbouring amplitudes, and the next tile bits are lane bits where the
+// planner could leave them, so a warp's loads fill 128-byte lines.  Against a
+// copy through shared memory this saves a tile's write there and a read, and
+// the copy's address arithmetic for every amplitude (400-step 14-spin ladder
+// 7.44 -> 7.15 ms, 40-step 18-spin one 6.3 -> 6.0; not used by the pipelined
+// sweep, whose compute groups would wait on their own loads and stores:
+// measured 8 to 20 % slower there).  Quads are walked in
+// Gray-code order over register bits 0 and 3..RB-1.
+__device__ __forceinline__ uint64_t direct_offset(uint64_t base, const uint8_t *thr, int tid, int lognt) {
+  uint64_t off = base;
+#pragma unroll
+  for (int b = 0; b < kMaxK - 5; ++b)
+    if (b < lognt && ((tid >> b) & 1)) off |= 1ull << thr[b];
+  return off;
+}
+// register index (quad's first amplitude) of Gray-code step g
+__host__ __device__ constexpr int quad_index(int g) { return ((g ^ (g >> 1)) & 1) | (((g ^ (g >> 1)) >> 1) << 3); }
+
+template <int RB>
+__device__ __forceinline__ void load_direct(const float2 *psi, uint64_t base, const PassDesc &d, int tid, int lognt,
+                                            u64 (&RE)[1 << (RB - 1)], u64 (&IM)[1 << (RB - 1)]) {
+  const char *src = reinterpret_cast<const char *>(psi + direct_offset(base, d.in_thr, tid, lognt));
+  int64_t dg[RB - 2];
+#pragma unroll
+  for (int k = 0; k < RB - 2; ++k) dg[k] = (int64_t)8 << d.in_reg[k ? k + 2 : 0];
+  u64 A[1 << RB];
+#pragma unroll
+  for (int g = 0; g < (1 << (RB - 2)); ++g) {
+    if (g) src += gray_up(g) ? dg[ctz5(g)] : -dg[ctz5(g)];
+    const int i = quad_index(g);
+    asm volatile("ld.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+                 : "=l"(A[i]), "=l"(A[i | 2]), "=l"(A[i | 4]), "=l"(A[i | 6])
+                 : "l"(src)
+                 : "memory");
+  }
+#pragma unroll
+  for (int j = 0; j < (1 << (RB - 1)); ++j) {
+    const float2 a = unpack2(A[2 * j]), b = unpack2(A[2 * j + 1]);
+    RE[j] = pack2(a.x, b.x);
+    IM[j] = pack2(a.y, b.y);
+  }
+}
+
+// The last phase's subcubes straight to the state, output tile bits 0 and 1
+// being register bits 1 and 2.
+template <int RB>
+__device__ __forceinline__ void store_direct(float2 *psi, uint64_t base, const PassDesc &d, int tid, int lognt,
+                                             const u64 (&RE)[1 << (RB - 1)], const u64 (&IM)[1 << (RB - 1)]) {
+  char *dst = reinterpret_cast<char *>(psi + direct_offset(base, d.out_thr, tid, lognt));
+  int64_t dg[RB - 2];
+#pragma unroll
+  for (int k = 0; k < RB - 2; ++k) dg[k] = (int64_t)8 << d.out_reg[k ? k + 2 : 0];
+#pragma unroll
+  for (int g = 0; g < (1 << (RB - 2)); ++g) {
+    if (g) dst += gray_up(g) ? dg[ctz5(g)] : -dg[ctz5(g)];
+    const int i = quad_index(g), j = i >> 1;
+    u64 v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 r = unpack2(RE[j | q]), m = unpack2(IM[j | q]);
+      v[q] = (i & 1) ? pack2(r.y, m.y) : pack2(r.x, m.x);
+    }
+    asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(v[0]), "l"(v[1]), "l"(v[2]), "l"(v[3])
+                 : "memory");
+  }
+}
+
 // The pass's phases on one tile in shared memory, run by the 2^lognt threads
-// tid of its group; `sync` is the group's barrier, sH/sQ/sOut the group's
-// diagonal-phase scratch, s_w the all-site scratch (SITES only).  ORIENT: the
-// program and the state are oriented (see Orientation).
-template <int RB, bool SITES, bool ORIENT, typename Sync>
+// tid of its group; `sync` is the group's barrier, sH the outer spins' fields
+// when the pass has a diagonal op (diag_fields), dtab its tables and s_w the
+// all-site scratch (SITES only).  ORIENT: the program and the state are oriented (see Orientation).
+// ENDS kDirect: RE/IM hold the first phase's subcubes (load_direct) and the last
+// phase goes to the state psi; kInPlace: the tile is in tile2 before and after.
+// WALK: rounds as walks over the register-bit pairs, else a jump to each gate
+// (the same gates in the same order).  DIAG: the pass may have a diagonal op.
+enum { kInPlace = 0, kDirect = 1 };
+template <int RB, bool SITES, bool ORIENT, int ENDS, bool WALK = true, bool DIAG = true, typename Sync>
 __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, const PhaseDesc *s_ph,
-                                           const ROpRes *s_op, uint64_t base, int tid, int lognt, int M,
-                                           const uint64_t *__restrict__ qdiag, float &up, float &dn,
-                                           uint64_t *sH, uint64_t *sQ, uint64_t *sOut, double *s_w,
-                                           Sync sync) {
-  constexpr int NA = 1 << RB, NP = NA / 2;
+                                           const ROpRes *s_op, uint64_t base, int tid, int lognt,
+                                           const uint64_t *__restrict__ dtab, float &up, float &dn,
+                                           const uint64_t *sH, double *s_w, Sync sync,
+                                           u64 (&RE)[1 << (RB - 1)], u64 (&IM)[1 << (RB - 1)], float2 *psi) {
+  constexpr int NP = 1 << (RB - 1);
   const uint32_t outer_par = ORIENT ? (uint32_t)(__popcll(base & d.black_outer) & 1) : 0u;
   for (int p = 0; p < d.nphases; ++p) {
     const PhaseDesc &ph = s_ph[p];
@@ -1242,8 +1395,9 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
 #pragma unroll
     for (int k = 0; k < RB; ++k) sm[k] = ph.sm[k];
     const int o0 = ph.op0 - d.rop0;
-    if (ph.nops == 1 && s_op[o0].kind == OP_DIAG) {
-      diag_phase<RB, ORIENT>(tile2, d, ph, s_op[o0], base, tid, lognt, M, qdiag, sH, sQ, sOut, s0, sm, sync);
+    if (DIAG && ph.nops == 1 && s_op[o0].kind == OP_DIAG) {
+      diag_tile<RB, ORIENT>(tile2, dtab + s_op[o0].tab, sH, d.K, tid, lognt, d.black_tile, outer_par);
+      sync();
       continue;
     }
     if constexpr (ORIENT) {
@@ -1253,13 +1407,12 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
     }
     // load the subcube as NP packs, walking the packs in Gray-code order so
     // each step changes one register bit (one XOR on the byte offset)
-    u64 RE[NP], IM[NP];
     const char *tb = reinterpret_cast<const char *>(tile2);
     uint32_t mb[RB];
 #pragma unroll
     for (int k = 0; k < RB; ++k) mb[k] = sm[k] << 3;
     const uint32_t ob = s0 << 3;
-    {
+    if (ENDS != kDirect || p > 0) {
       uint32_t o = ob;
 #pragma unroll
       for (int g = 0; g < NP; ++g) {
@@ -1279,11 +1432,15 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
         IM[j] = pack2(v0.y, v1.y);
       }
     }
-    ROpRes cur = s_op[o0];
     for (int k = 0; k < ph.nops; ++k) {
-      const ROpRes nxt = s_op[o0 + (k + 1 < ph.nops ? k + 1 : k)];  // prefetch
-      if (cur.kind == OP_GATE) {
+      const ROpRes cur = s_op[o0 + k];
+      if (!WALK && cur.kind == OP_GATE) {
         gate_combo(RE, IM, cur.combo, cur.t, cur.s);
+      } else if (WALK && cur.kind == OP_ROUND) {
+        const ROpRes *first = s_op + o0 + k + 1;
+        const float2 ts = make_float2(first->t, first->s);
+        run_round<NP>(RE, IM, cur.tab, first, ts);
+        k += cur.arg;
       } else if (cur.kind == OP_REDUCE) {
         int kr = -1;
 #pragma unroll
@@ -1340,9 +1497,12 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
           warp_site_sum<float>(tsum, kMaxK, s_w);
         }
       }
-      cur = nxt;
     }
-    {
+    if (ENDS == kDirect && p == d.nphases - 1) {
+      // one phase only: every load of the tile before its relabelled stores
+      if (p == 0) sync();
+      store_direct<RB>(psi, base, d, tid, lognt, RE, IM);
+    } else {
       char *tw = reinterpret_cast<char *>(tile2);
       uint32_t o = ob;
 #pragma unroll
@@ -1419,8 +1579,9 @@ __device__ __forceinline__ void store_tile(float2 *psi, uint64_t base, const Pas
 
 // Register-blocked sweep with RB register bits (2^RB amplitudes per thread,
 // 2^(K-RB) threads per tile), one tile per block.  ORIENT: an oriented
-// program on an oriented state (see Orientation).
-template <int RB, bool SITES, bool ORIENT>
+// program on an oriented state (see Orientation).  DIRECT: a direct pass, whose
+// first and last phase move the tile between registers and the state.
+template <int RB, bool SITES, bool ORIENT, bool DIRECT>
 __global__ void __launch_bounds__(RB == 5 ? 512 : 256)
 sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops1,
               const __grid_constant__ PassDesc d, const PhaseDesc *__restrict__ phases, int M,
@@ -1432,11 +1593,9 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   const JobPtrs jp = jobs[blockIdx.y];
   float2 *__restrict__ psi = one ? psi1 : static_cast<float2 *>(jp.psi);
   extern __shared__ __align__(16) float2 tile2[];
-  __shared__ uint64_t sH[kMaxK];
-  __shared__ uint64_t sQ[kMaxK * kMaxK];
-  __shared__ uint64_t sOut;
+  __shared__ uint64_t sH[kMaxK + 1];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
-  __shared__ __align__(16) ROpRes s_op[kMaxPassOps];
+  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 1];  // a round reads one coefficient ahead
   __shared__ double s_w[SITES ? kMaxWarps * kSiteSlots : 1];
   const int tid = threadIdx.x, nt = blockDim.x;
   const int lognt = d.K - RB;
@@ -1445,7 +1604,9 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   // resolved for this dt), then the L2 prefetch of the tile of block
   // blockIdx.x + ahead (ahead = blocks resident at once): DRAM keeps
   // streaming while tiles compute, and that block's copies find its tile in L2
-  sw2::load_tile<RB>(psi, base, d, tid, lognt, (uint32_t)__cvta_generic_to_shared(tile2));
+  sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
+  if constexpr (DIRECT) sw2::load_direct<RB>(psi, base, d, tid, lognt, RE, IM);
+  else sw2::load_tile<RB>(psi, base, d, tid, lognt, (uint32_t)__cvta_generic_to_shared(tile2));
   {
     const uint32_t *pw = reinterpret_cast<const uint32_t *>(phases + d.phase0);
     const uint32_t a_ph = (uint32_t)__cvta_generic_to_shared(s_ph);
@@ -1457,13 +1618,14 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   }
   if (ahead && blockIdx.x + ahead < gridDim.x)
     sw2::prefetch_tile<RB>(psi, sw2::tile_origin(blockIdx.x + ahead, d, M), d, tid, lognt);
+  if (d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   sw2::cp_async_wait_all();
   __syncthreads();
 
   float up = 0.f, dn = 0.f;
-  sw2::run_phases<RB, SITES, ORIENT>(tile2, d, s_ph, s_op, base, tid, lognt, M, jp.qdiag, up, dn, sH, sQ,
-                                     &sOut, s_w, sw2::SyncBlock{});
-  sw2::store_tile<RB>(psi, base, d, tid, lognt, tile2);
+  sw2::run_phases<RB, SITES, ORIENT, DIRECT ? sw2::kDirect : sw2::kInPlace>(tile2, d, s_ph, s_op, base, tid, lognt, jp.dtab, up, dn, sH, s_w,
+                                             sw2::SyncBlock{}, RE, IM, psi);
+  if constexpr (!DIRECT) sw2::store_tile<RB>(psi, base, d, tid, lognt, tile2);
   if constexpr (SITES)
     if (d.has_reduce) write_site_partials(d, M, base, s_w, jp.psites);
   if (d.has_reduce) reduce_finalize((double)up, (double)dn, jp, false);
@@ -1494,9 +1656,7 @@ resident_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ Reside
   extern __shared__ __align__(16) float2 tile2[];
   PhaseDesc *s_ph = reinterpret_cast<PhaseDesc *>(tile2 + (size_t(1) << M));
   ROpRes *s_op = reinterpret_cast<ROpRes *>(s_ph + nph);
-  __shared__ uint64_t sH[kMaxK];
-  __shared__ uint64_t sQ[kMaxK * kMaxK];
-  __shared__ uint64_t sOut;
+  __shared__ uint64_t sH[kMaxK + 1];
   __shared__ double s_up[8], s_dn[8];
   const int tid = threadIdx.x, nt = blockDim.x;
   const int lognt = M - RB;
@@ -1510,6 +1670,7 @@ resident_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ Reside
     const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
     for (int i = tid; i < nrops; i += nt) sw2::cp_async16(a_op + 16u * i, jp.sops + i);
   }
+  for (int i = tid; i <= M; i += nt) sH[i] = 0;  // no outer spins: no fields
   sw2::cp_async_wait_all();
   __syncthreads();
   const int64_t slot0 = *jp.step;
@@ -1517,8 +1678,9 @@ resident_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ Reside
   for (int64_t k = 0; k < steps; ++k) {
     const PassDesc &d = steps == 1 ? rp.only : k == 0 ? rp.first : k == steps - 1 ? rp.last : rp.mid;
     float up = 0.f, dn = 0.f;
-    sw2::run_phases<RB, false, ORIENT>(tile2, d, s_ph + d.phase0, s_op + d.rop0, 0ull, tid, lognt, M,
-                                       jp.qdiag, up, dn, sH, sQ, &sOut, nullptr, sw2::SyncBlock{});
+    sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
+    sw2::run_phases<RB, false, ORIENT, sw2::kInPlace>(tile2, d, s_ph + d.phase0, s_op + d.rop0, 0ull, tid, lognt, jp.dtab,
+                                              up, dn, sH, nullptr, sw2::SyncBlock{}, RE, IM, nullptr);
     // this step's N_up / N_dn: FP64 sums over the block in a fixed order
     double u = up, w = dn;
     for (int o = 16; o; o >>= 1) {

@@ -177,11 +177,9 @@ __global__ void __launch_bounds__(256)
 persist_kernel(const PersistPlan *__restrict__ plan, unsigned long long *queue, unsigned *done, int *err,
                unsigned ahead) {
   extern __shared__ __align__(16) float2 tile2[];
-  __shared__ uint64_t sH[kMaxK];
-  __shared__ uint64_t sQ[kMaxK * kMaxK];
-  __shared__ uint64_t sOut;
+  __shared__ uint64_t sH[kMaxK + 1];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
-  __shared__ __align__(16) ROpRes s_op[kMaxPassOps];
+  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 1];  // a round reads one coefficient ahead
   __shared__ __align__(16) PassDesc s_d;
   __shared__ double s_up[8], s_dn[8];
   __shared__ unsigned long long s_item;
@@ -275,11 +273,13 @@ persist_kernel(const PersistPlan *__restrict__ plan, unsigned long long *queue, 
     if (ahead && r + ahead < G.tiles) sw2::prefetch_tile<RB>(psi, sw2::tile_origin(r + ahead, d, M), d, tid, lognt);
     pq::load_tile_cg<RB>(psi, base, d, tid, lognt, tile2);
     if (tid == 0) next = atomicAdd(queue, 1ull);
+    if (d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
     sw2::cp_async_wait_all();
     __syncthreads();
     float up = 0.f, dn = 0.f;
-    sw2::run_phases<RB, false, false>(tile2, d, s_ph, s_op, base, tid, lognt, M, jp.qdiag, up, dn, sH, sQ,
-                                      &sOut, nullptr, sw2::SyncBlock{});
+    sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
+    sw2::run_phases<RB, false, false, sw2::kInPlace>(tile2, d, s_ph, s_op, base, tid, lognt, jp.dtab, up, dn, sH, nullptr,
+                                             sw2::SyncBlock{}, RE, IM, nullptr);
     sw2::store_tile<RB>(psi, base, d, tid, lognt, tile2);
     if (d.has_reduce) pq::reduce_tile((double)up, (double)dn, jp, r, G.tiles, s_up, s_dn, &s_last);
     __threadfence();

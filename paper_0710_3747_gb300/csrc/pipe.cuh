@@ -156,11 +156,11 @@ __device__ __forceinline__ void pipe_finalize(const double2 *partials, unsigned 
 // sweep2_kernel's readout variant: under this kernel's 224-register budget
 // the readout's sums spill, measured 8 % slower per step at M = 30.)
 //   BATCH = false: one job; jobs[0] holds its pointers (gate tables,
-//     partials, ticket, series), psi1 and sops1 its amplitudes and resolved
-//     ops; the units are its tiles, and the last block to finish combines
+//     partials, ticket, series), psi1, sops1, qdiag1 and dtab1 its amplitudes,
+//     resolved ops and diagonal-phase tables; the units are its tiles, and the last block to finish combines
 //     the tile partials.
-//   BATCH = true: njobs jobs of the same plan (jobs[j]), job j's amplitudes
-//     and resolved ops at psi1 and sops1 plus j x jstride bytes; the units
+//   BATCH = true: njobs jobs of the same plan (jobs[j]), job j's amplitudes,
+//     resolved ops and tables at those addresses plus j x jstride bytes; the units
 //     are the (job, tile) pairs, job-major; the producer copies each unit's job
 //     pointers and resolved ops (at most kPipeBatchOps) into its buffer's
 //     slots of static shared arrays with the tile (the same mbarrier covers
@@ -170,25 +170,32 @@ __device__ __forceinline__ void pipe_finalize(const double2 *partials, unsigned 
 // runs out (the check that the waits are bounded; nothing is written to the
 // amplitudes or the series).  Dynamic shared memory: three 8 x 2^K byte tile
 // buffers.
+// VAR: passes with the diagonal op (kPipeDiag), and of the others the ones with
+// many gates a phase (kPipeDense: walks over the register-bit pairs) and with
+// few (kPipeSparse: a jump to each gate's code; most pairs of a walk would be
+// skipped, and the whole walk's code competes for the instruction cache with
+// the producer's).  Measured with walks against jumps: 25-spin dipolar star
+// (8.7 gates a phase) 18.3 against 21.8 ms for six steps, 26-spin ladder (5.4)
+// 24.5 against 22.5 ms for twenty; the line lies between.
+constexpr int kPipeDenseGates = 7;
+enum { kPipeSparse = 0, kPipeDense = 1, kPipeDiag = 2 };
 constexpr int kPipeBatchOps = kMaxPassOps / 3;  // resolved ops of a pass, per buffer (batches)
 static_assert(sizeof(JobPtrs) % 8 == 0, "job pointers copied as 8-byte words");
 
-template <int RB, int K, bool BATCH>
+template <int RB, int K, bool BATCH, int VAR>
 __global__ void __launch_bounds__(kPipeThreads, 1)
-pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROpRes *sops1, long long jstride,
-            const __grid_constant__ PassDesc d, const PhaseDesc *__restrict__ phases, int M, int *err, int probe) {
+pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROpRes *sops1,
+            const uint64_t *qdiag1, const uint64_t *dtab1, long long jstride, const __grid_constant__ PassDesc d, const PhaseDesc *__restrict__ phases, int M, int *err, int probe) {
   constexpr int LOGNT = K - RB;
   constexpr int NT = 1 << LOGNT;   // threads of a group (a warpgroup)
   constexpr int NW = NT / 32;      // warps of a group
   constexpr uint32_t TA = 1u << K; // amplitudes per tile buffer
   static_assert(NT == 128, "groups are warpgroups");
   extern __shared__ __align__(16) float2 tiles[];
-  __shared__ uint64_t sH[2][kMaxK];
-  __shared__ uint64_t sQ[2][kMaxK * kMaxK];
-  __shared__ uint64_t sOut[2];
+  __shared__ uint64_t sH[2][kMaxK + 1];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
   // one job: the pass's ops; BATCH: three slices of kPipeBatchOps, one per buffer
-  __shared__ __align__(16) ROpRes s_op[kMaxPassOps];
+  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 1];  // a round reads one coefficient ahead
   __shared__ __align__(16) JobPtrs s_job[BATCH ? 3 : 1];
   __shared__ __align__(8) uint64_t s_full[3], s_done[3];
   __shared__ double s_up[2][NW], s_dn[2][NW];
@@ -283,21 +290,29 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
   const pipe::SyncNamed sync{bar, (uint32_t)NT};
   for (unsigned i = (unsigned)g; i < nloc; i += 2u) {
     const uint32_t b = i % 3u;
+    const unsigned u = blockIdx.x + i * G;
+    const unsigned tile = u & (T - 1u);
+    const uint64_t base = sw2::tile_origin(tile, d, M);
+    // the tile's outer fields while its amplitudes are on their way; the
+    // barrier after the wait publishes them
+    const long long joff = BATCH ? (long long)(u >> lt) * jstride : 0;
+    const uint64_t *const qdiag =
+        reinterpret_cast<const uint64_t *>(reinterpret_cast<const char *>(qdiag1) + joff);
+    const uint64_t *const dtab = reinterpret_cast<const uint64_t *>(reinterpret_cast<const char *>(dtab1) + joff);
+    if (VAR == kPipeDiag && !probe) sw2::diag_fields(d, base, gt, LOGNT, M, qdiag, sH[g]);
     const bool late = !pipe::mbar_wait(a_full + 8u * b, (i / 3u) & 1u, err);
     if (pipe::group_any(late, bar, NT)) {
       if (gt == 0) atomicExch(err, 1);
       break;
     }
-    const unsigned u = blockIdx.x + i * G;
-    const unsigned tile = u & (T - 1u);
     // the unit's job pointers: BATCH from its buffer's slot, which stays
     // valid until the buffer is handed back
     const JobPtrs *js = BATCH ? &s_job[b] : jobs;
     const ROpRes *ops = BATCH ? s_op + kPipeBatchOps * b : s_op;
-    const uint64_t base = sw2::tile_origin(tile, d, M);
     float up = 0.f, dn = 0.f;
-    sw2::run_phases<RB, false, false>(tiles + b * TA, d, s_ph, ops, base, gt, LOGNT, M, js->qdiag, up, dn, sH[g],
-                                      sQ[g], &sOut[g], nullptr, sync);
+    sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
+    sw2::run_phases<RB, false, false, sw2::kInPlace, VAR != kPipeSparse, VAR == kPipeDiag>(
+        tiles + b * TA, d, s_ph, ops, base, gt, LOGNT, dtab, up, dn, sH[g], nullptr, sync, RE, IM, nullptr);
     // run_phases ends with the group's barrier: the tile is finished
     if (!d.has_reduce) {
       if (gt == 0) pipe::mbar_arrive(a_done + 8u * b);

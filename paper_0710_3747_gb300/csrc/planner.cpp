@@ -193,7 +193,9 @@ bool build_plan(int M, const std::vector<std::pair<int, int>> &bonds, int K, int
     for (int q = 0; q < M; ++q)
       if ((Q >> q) & 1) qs.push_back(q);
     plan->segQ.push_back(qs);
-    // exit set: the c spins of Q whose next pending gate comes earliest
+    // exit set: the c spins of Q whose next pending gate comes earliest, in that
+    // order (the next segment starts with the first ones, and its reverse ends
+    // with them: direct passes hold low bits 0 and 1 in those phases)
     std::vector<std::pair<long, int>> cand;
     for (int q : qs) {
       const int h = fr.head(q);
@@ -201,8 +203,7 @@ bool build_plan(int M, const std::vector<std::pair<int, int>> &bonds, int K, int
     }
     std::sort(cand.begin(), cand.end());
     std::vector<int> X;
-    for (int k = 0; k < c; ++k) X.push_back(cand[k].second);
-    std::sort(X.begin(), X.end());
+    for (int k = 0; k < c; ++k) X.push_back(cand[k].second);  // the earliest first: low bits 0, 1, ...
     plan->exitX.push_back(X);
     entry = 0;
     for (int q : X) entry |= 1ull << q;
@@ -301,7 +302,7 @@ static void for_each_subset(const std::vector<int> &items, int take, F f) {
 
 bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, int beam, int fence,
                  std::vector<uint32_t> *sets, std::vector<std::vector<int>> *applied, uint32_t black,
-                 uint32_t nb_allowed) {
+                 uint32_t nb_allowed, const PhaseEnds &ends) {
   sets->clear();
   applied->clear();
   const int n = (int)gates.size();
@@ -319,6 +320,20 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
   BitPtr zero;
   zero.fill(0);
   levels[0].push_back(PhaseState{zero, 0, 0, -1, 0});
+  // a set of RB bits from R: idle bits added, the last set's first, the ones
+  // to avoid last
+  const uint32_t all = (1u << K) - 1u;
+  auto pad = [&](uint32_t R, uint32_t avoid) {
+    for (uint32_t pool : {ends.last, all & ~avoid, all})
+      for (int q = 0; q < K && __builtin_popcount(R) < RB; ++q)
+        if ((pool >> q) & 1u) R |= 1u << q;
+    return R;
+  };
+  auto penalty = [&](const PhaseState &s, int depth) {
+    int p = depth == 0 ? __builtin_popcount(s.set & ends.avoid_first) : 0;
+    if (s.done == n) p += (s.set & ends.last) == ends.last ? __builtin_popcount(s.set & ends.avoid_last) : 8;
+    return p;
+  };
   for (int depth = 0; depth < 4 * n + 4; ++depth) {
     const std::vector<PhaseState> &cur = levels.back();
     std::vector<PhaseState> next;
@@ -338,11 +353,20 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
         }
       };
       if (nb_allowed == 0) {
-        const int take = std::min<int>(RB, (int)live.size());
-        for_each_subset(live, take, [&](uint32_t R) {
-          for (int q = 0; q < K && __builtin_popcount(R) < RB; ++q) R |= 1u << q;
-          try_set(R);
-        });
+        // the first set holds ends.first; a set that may be the last one is
+        // also tried with ends.last
+        const uint32_t must = depth == 0 ? ends.first : 0u;
+        const uint32_t avoid = (depth == 0 ? ends.avoid_first : 0u) | ends.avoid_last;
+        for (uint32_t base : {must, must | ends.last}) {
+          const int room = RB - __builtin_popcount(base);
+          if (room < 0) continue;
+          std::vector<int> pick;
+          for (int q : live)
+            if (!((base >> q) & 1u)) pick.push_back(q);
+          for_each_subset(pick, std::min<int>(room, (int)pick.size()),
+                          [&](uint32_t R) { try_set(pad(base | R, avoid)); });
+          if (ends.last == 0 || (must | ends.last) == must) break;
+        }
       } else {
         // for each allowed count nb: nb live bits of the colour `black` and
         // RB - nb of the other (fewer when fewer are live), each side padded
@@ -368,8 +392,9 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
     }
     if (next.empty()) return false;
     // keep the `beam` best distinct states (most gates done)
-    std::stable_sort(next.begin(), next.end(),
-                     [](const PhaseState &a, const PhaseState &b) { return a.done > b.done; });
+    std::stable_sort(next.begin(), next.end(), [&](const PhaseState &a, const PhaseState &b) {
+      return a.done != b.done ? a.done > b.done : penalty(a, depth) < penalty(b, depth);
+    });
     std::vector<PhaseState> kept;
     for (PhaseState &c : next) {
       bool dup = false;
@@ -398,10 +423,80 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
         sets->push_back(R);
         applied->push_back(out);
       }
+      if ((sets->back() & ends.last) != ends.last) {
+        sets->push_back(pad(ends.last, ends.avoid_last));
+        applied->push_back({});
+      }
       return true;
     }
   }
   return false;
+}
+
+// ---------------------------------------------------------------------------
+// Rounds of a phase (see PhaseRound).
+// ---------------------------------------------------------------------------
+namespace {
+
+// Rounds of gates [from, to) under the labelling ku < kv (combo: the pair's
+// index); returns their number and writes them when out is non-null.
+int greedy_rounds(const std::vector<int> &ku, const std::vector<int> &kv, const std::vector<int> &combo, int RB,
+                  int from, int to, std::vector<PhaseRound> *out) {
+  std::array<std::vector<int>, kMaxRegBits> chain;  // per register bit: its gates in order
+  std::array<size_t, kMaxRegBits> ptr{};
+  for (int g = from; g < to; ++g) chain[ku[g]].push_back(g), chain[kv[g]].push_back(g);
+  int n = 0;
+  for (int left = to - from; left > 0; ++n) {
+    PhaseRound r;
+    for (int u = 0; u < RB; ++u)
+      for (int v = u + 1; v < RB; ++v)
+        if (ptr[u] < chain[u].size() && ptr[v] < chain[v].size() && chain[u][ptr[u]] == chain[v][ptr[v]]) {
+          r.gates.push_back(chain[u][ptr[u]]);
+          ++ptr[u], ++ptr[v];
+        }
+    left -= (int)r.gates.size();
+    r.combo = combo;
+    if (out) out->push_back(r);
+  }
+  return n;
+}
+
+}  // namespace
+
+void plan_rounds(const std::vector<std::pair<int, int>> &gates, int RB, int split, int fix1, int fix2,
+                 std::vector<int> *rb, std::vector<PhaseRound> *rounds) {
+  const int n = (int)gates.size();
+  std::vector<int> order = *rb, best_order;  // order[k]: tile bit of register bit k
+  std::sort(order.begin(), order.end());
+  std::vector<int> ku(n), kv(n), combo(n), idx(kMaxK);
+  auto label = [&]() {
+    for (int k = 0; k < RB; ++k) idx[order[k]] = k;
+    int pack = 0;
+    for (int g = 0; g < n; ++g) {
+      const int a = idx[gates[g].first], b = idx[gates[g].second];
+      ku[g] = std::min(a, b), kv[g] = std::max(a, b);
+      combo[g] = ku[g] * (2 * RB - ku[g] - 1) / 2 + kv[g] - ku[g] - 1;
+      pack += ku[g] == 0;
+    }
+    return pack;
+  };
+  const int cut = split < 0 ? 0 : split;
+  // a gate on the pack bit costs a gate more, a round about two (its tests)
+  int best = std::numeric_limits<int>::max();
+  do {
+    if ((fix1 >= 0 && order[1] != fix1) || (fix2 >= 0 && order[2] != fix2)) continue;
+    const int pack = label();
+    if (pack >= best) continue;
+    const int r = greedy_rounds(ku, kv, combo, RB, 0, cut, nullptr) + greedy_rounds(ku, kv, combo, RB, cut, n, nullptr);
+    if (pack + 2 * r < best) best = pack + 2 * r, best_order = order;
+  } while (std::next_permutation(order.begin(), order.end()));
+  order = best_order;
+  label();
+  *rb = order;
+  rounds->clear();
+  greedy_rounds(ku, kv, combo, RB, 0, cut, rounds);
+  if (split >= 0) rounds->push_back(PhaseRound{});
+  greedy_rounds(ku, kv, combo, RB, cut, n, rounds);
 }
 
 }  // namespace spinrp
