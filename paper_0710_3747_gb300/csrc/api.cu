@@ -1571,12 +1571,30 @@ static int launch_resident(const LaunchCtx &c, cudaStream_t stream, int64_t step
   return SPINRP_OK;
 }
 
+// A sweep launch.  chained: it may start while the kernel before it on the
+// stream, a sweep too, still runs; the kernel stages its program and waits for
+// that one before it touches the state (grid_wait).  Not for the first sweep of
+// an evolve call: the tables it stages may have just been launched.  Takes part
+// of a sweep's launch and prologue off the chain (per step: 14-spin ladder 17.9
+// -> 16.9 us, complex128 37.7 -> 35.6; 17-spin star 62.3 -> 59.5).
+template <typename... P, typename... A>
+static cudaError_t launch_sweep(bool chained, dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
+                                void (*kernel)(P...), A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid, cfg.blockDim = dim3(threads), cfg.dynamicSmemBytes = smem, cfg.stream = stream;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr, cfg.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Launch one sweep on `stream`; `live` launches are counted and profiled,
 // launches recorded into a graph are not.
 template <typename R>
-static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool live) {
+static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool live, bool chained) {
   const int K = c.K;
-  const int nt = std::min(512, std::max(32, 1 << K));
+  const int nt = std::min(512, std::max(32, 1 << K >> 1));  // plain sweep: a thread a plane
   const size_t smem = sizeof(typename CT<R>::T) << K;
   const dim3 grid(1u << (c.M - K), (unsigned)c.njobs);
   if (live) {
@@ -1586,6 +1604,11 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
   // the all-site sums are taken only in the sweep that reads P out; the
   // other sweeps of an all-site run are the plain ones
   const bool sites = c.sites && c.ps->desc[pass].has_reduce;
+  // one-tile-per-block sweeps of more blocks than SMs start after the sweep
+  // before: blocks let in early land where that one's blocks are not, and stay
+  // unevenly spread (20-spin star, 256 blocks: 160 us a step against 113).
+  // (At most two complex128 tiles share an SM: 138 us a sweep against 140.)
+  const bool few = (uint64_t)grid.x * grid.y <= (uint64_t)kModelSMs || sizeof(R) == 8;
   if (sizeof(R) == 4 && c.v2)
   {
     const size_t sm2 = size_t(8) << K;
@@ -1596,10 +1619,10 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
     const int code = (c.rb == 6 ? 4 : 0) | (sites ? 2 : 0) | (c.oriented ? 1 : 0);
     const bool piped = c.pipe_blocks && K == 13 && code == 4;
     if (piped) {
-#define PIPE(B_, V_)                                                                                         \
-  pipe_kernel<6, 13, B_, V_><<<c.pipe_blocks, kPipeThreads, kPipeSmem, stream>>>(                            \
-      c.jobs, c.njobs, static_cast<float2 *>(j0.psi), j0.sops, j0.qdiag, j0.dtab, B_ ? c.job_stride : 0, pd, \
-      c.phases, c.M, c.pipe_err, 0)
+#define PIPE(B_, V_)                                                                                             \
+  CUDA_TRY(launch_sweep(chained, dim3(c.pipe_blocks), kPipeThreads, kPipeSmem, stream, pipe_kernel<6, 13, B_, V_>, \
+                        c.jobs, c.njobs, static_cast<float2 *>(j0.psi), j0.sops, j0.qdiag, j0.dtab,               \
+                        B_ ? c.job_stride : 0ll, pd, c.phases, c.M, c.pipe_err, 0))
       const JobPtrs &j0 = c.njobs == 1 ? c.job0 : c.batch0;
       const bool many = c.njobs > 1;
       switch (2 * c.ps->variant(pass) + (many ? 1 : 0)) {
@@ -1617,8 +1640,9 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
         pipe_finalize_kernel<<<c.njobs, 128, 0, stream>>>(c.jobs, 1u << (c.M - 13), c.pipe_err);
       }
     } else {
-#define SW2(RB_, S_, O_, D_) \
-  sweep2_kernel<RB_, S_, O_, D_><<<grid, 1 << (K - RB_), sm2, stream>>>(c.jobs, psi1, sops1, pd, c.phases, c.M, ahead)
+#define SW2(RB_, S_, O_, D_)                                                                          \
+  CUDA_TRY(launch_sweep(chained && few, grid, 1u << (K - RB_), sm2, stream, sweep2_kernel<RB_, S_, O_, D_>, c.jobs, \
+                        psi1, sops1, pd, c.phases, c.M, ahead, chained && few))
       switch (code | (pd.direct ? 8 : 0)) {
         case 0: SW2(5, false, false, false); break;
         case 1: SW2(5, false, true, false); break;
@@ -1638,12 +1662,12 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
   }
   else if (sizeof(R) == 8 && c.v2 && !sites)
     // complex128 register-blocked (the all-site sums run in the plain kernel)
-    sweep2d_kernel<<<grid, 1 << (K - 5), smem, stream>>>(c.jobs, c.ps->desc[pass], c.phases, c.rops, c.M,
-                                                          c.prefetch_ahead);
+    CUDA_TRY(launch_sweep(chained && few, grid, 1u << (K - 5), smem, stream, sweep2d_kernel, c.jobs, c.ps->desc[pass], c.phases,
+                          c.rops, c.M, c.prefetch_ahead));
   else if (sites)
-    sweep_kernel<R, true><<<grid, nt, smem, stream>>>(c.jobs, c.passes + pass, c.ops, c.M);
+    CUDA_TRY(launch_sweep(chained && few, grid, nt, smem, stream, sweep_kernel<R, true>, c.jobs, c.passes + pass, c.ops, c.M));
   else
-    sweep_kernel<R, false><<<grid, nt, smem, stream>>>(c.jobs, c.passes + pass, c.ops, c.M);
+    CUDA_TRY(launch_sweep(chained && few, grid, nt, smem, stream, sweep_kernel<R, false>, c.jobs, c.passes + pass, c.ops, c.M));
   CUDA_TRY(cudaGetLastError());
   if (c.sites && c.ps->desc[pass].has_reduce) {
     if (live) ++g_launches;
@@ -1654,9 +1678,9 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
   return SPINRP_OK;
 }
 
-#define RUN(pass)                                           \
-  do {                                                      \
-    int rc_ = launch_pass<R>(c, (pass), stream, live);      \
+#define RUN(pass)                                                   \
+  do {                                                              \
+    int rc_ = launch_pass<R>(c, (pass), stream, live, chained);     \
     if (rc_) return rc_;                                    \
   } while (0)
 
@@ -1665,6 +1689,7 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
 template <typename R>
 static int steady_steps(const LaunchCtx &c, cudaStream_t stream, int64_t n, bool live) {
   const PassSet &ps = *c.ps;
+  const bool chained = true;
   for (int64_t k = 0; k < n; ++k) {
     if (c.segments == 1) {
       RUN(ps.midstep);
@@ -1683,6 +1708,7 @@ static int steady_steps(const LaunchCtx &c, cudaStream_t stream, int64_t n, bool
 template <typename R>
 static int first_step(const LaunchCtx &c, cudaStream_t stream, int64_t steps, bool live) {
   const PassSet &ps = *c.ps;
+  const bool chained = false;
   if (c.segments == 1) RUN(steps == 1 ? ps.only : ps.first);
   else RUN(ps.head);
   return SPINRP_OK;
@@ -1691,6 +1717,7 @@ static int first_step(const LaunchCtx &c, cudaStream_t stream, int64_t steps, bo
 template <typename R>
 static int last_step(const LaunchCtx &c, cudaStream_t stream, int64_t steps, bool live) {
   const PassSet &ps = *c.ps;
+  const bool chained = true;
   if (c.segments == 1) {
     if (steps > 1) RUN(ps.last);
   } else {

@@ -169,7 +169,7 @@ struct JobPtrs {
 
 // Gate coefficients of exp(-i theta sigma_x) on a flip-flop pair, theta = b tau/2:
 // (tan theta/2, sin theta) of the three-shear form of the two real plane
-// rotations the gate is made of (see shear_rotate), in FP64 and as the FP32
+// rotations the gate is made of (see shear_plane), in FP64 and as the FP32
 // pair closest to a rotation.
 struct GateCoef {
   double t, s;

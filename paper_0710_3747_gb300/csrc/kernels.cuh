@@ -27,6 +27,14 @@ struct LayoutArg {
   uint8_t logical_of[kMaxM];  // physical bit position -> logical spin
 };
 
+// Sweeps follow each other with programmatic dependences: a sweep's blocks may
+// be resident, with the pass's program staged (it does not depend on the sweep
+// before), while that sweep still runs; grid_wait() returns once every earlier
+// kernel has finished and its writes are visible, grid_go() lets the next
+// sweep's blocks in as soon as all of this one's are (see launch_sweep).
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ uint64_t deposit_bits(uint64_t v, const uint8_t *pos, int n) {
   uint64_t r = 0;
   for (int k = 0; k < n; ++k) r |= ((v >> k) & 1ull) << pos[k];
@@ -482,51 +490,70 @@ __global__ void diag_tab_kernel(const JobPtrs *__restrict__ jobs, const __grid_c
 // x += t y with t = tan(theta/2): three FMAs per plane.  A shear has
 // determinant one whatever t and s are rounded to, so rounding leaves no
 // uniform gain or loss of norm.
-__device__ __forceinline__ void shear_rotate(float2 &a, float2 &b, float t, float s) {
-  float x = fmaf(t, b.y, a.x);
-  b.y = fmaf(-s, x, b.y);
-  a.x = fmaf(t, b.y, x);
-  x = fmaf(t, a.y, b.x);
-  a.y = fmaf(-s, x, a.y);
-  b.x = fmaf(t, a.y, x);
+__device__ __forceinline__ void shear_plane(float &x, float &y, float t, float s) {
+  const float v = fmaf(t, y, x);
+  y = fmaf(-s, v, y);
+  x = fmaf(t, y, v);
 }
-__device__ __forceinline__ void shear_rotate(double2 &a, double2 &b, double t, double s) {
-  double x = fma(t, b.y, a.x);
-  b.y = fma(-s, x, b.y);
-  a.x = fma(t, b.y, x);
-  x = fma(t, a.y, b.x);
-  a.y = fma(-s, x, a.y);
-  b.x = fma(t, a.y, x);
+__device__ __forceinline__ void shear_plane(double &x, double &y, double t, double s) {
+  const double v = fma(t, y, x);
+  y = fma(-s, v, y);
+  x = fma(t, y, v);
 }
 
+// The plain sweep: tiles below ten spins, and the complex128 all-site readout.
+// A gate takes the tile's pairs from shared memory, real and imaginary parts
+// apart, one thread a plane (half the FP64 chain, and twice the warps, of a
+// thread a pair), with the pass's ops and coefficients staged there first.  A
+// 14-spin complex128 sweep is bound by its gates' latency: 0.75 us a gate with
+// op and coefficients read from global memory at each gate and both planes in
+// one thread, 0.45 us so (the 26-gate sweep 23 -> 18 us with its launch, the
+// 400-step job 15.0 -> 10.3 ms with the sweeps chained too).
+constexpr int kMaxPlainOps = 192;  // every pair of 14 tile bits twice, and the element-wise ops
+static_assert(kMaxK * (kMaxK - 1) + 4 <= kMaxPlainOps, "ops of a pass");
 
 template <typename R, bool SITES>
 __global__ void __launch_bounds__(512)
 sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdesc,
              const Op *__restrict__ ops, int M) {
   using C = typename CT<R>::T;
+  struct SOp {
+    uint8_t kind, u, v, arg;
+    R t, s;
+  };
   const JobPtrs jp = jobs[blockIdx.y];
   C *__restrict__ psi = static_cast<C *>(jp.psi);
-  const GateCoef *__restrict__ coefs = jp.coefs;
   const uint64_t *__restrict__ qdiag = jp.qdiag;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C *tile = reinterpret_cast<C *>(smem_raw);
   __shared__ PassDesc d;
   __shared__ uint64_t sH[kMaxK];
   __shared__ uint64_t sQ[kMaxK * kMaxK];
   __shared__ uint64_t sOut;
   __shared__ double s_w[SITES ? kMaxWarps * kSiteSlots : 1];
+  __shared__ SOp s_ops[kMaxPlainOps];
+  grid_go();
   {
     const int nwords = (int)(sizeof(PassDesc) / 4);
     for (int w = threadIdx.x; w < nwords; w += blockDim.x)
       reinterpret_cast<int *>(&d)[w] = reinterpret_cast<const int *>(pdesc)[w];
   }
   __syncthreads();
+  for (int k = threadIdx.x; k < d.nops; k += blockDim.x) {
+    const Op op = ops[d.op0 + k];
+    SOp o{op.kind, op.u, op.v, op.arg, 0, 0};
+    if (op.kind == OP_GATE) {
+      const GateCoef g = jp.coefs[op.coef];
+      o.t = sizeof(R) == 8 ? (R)g.t : (R)g.tf;
+      o.s = sizeof(R) == 8 ? (R)g.s : (R)g.sft;
+    }
+    s_ops[k] = o;
+  }
   const int K = d.K;
   const int nt = blockDim.x, tid = threadIdx.x;
   const int lognt = 31 - __clz(nt);
   const int L = lognt < K ? lognt : K;  // tile bits taken from the thread index
   const uint32_t T = 1u << K;
+  R *const re = reinterpret_cast<R *>(smem_raw), *const im = re + T;
   const uint64_t base = deposit_bits(blockIdx.x, d.outer_pos, M - K);
   const uint64_t off_lo = deposit_bits(tid, d.tile_pos, L);
   auto offset = [&](uint32_t t) -> uint64_t {
@@ -534,24 +561,27 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
     for (int q = L; q < K; ++q) o |= (uint64_t)((t >> q) & 1u) << d.tile_pos[q];
     return o;
   };
-  for (uint32_t t = tid; t < T; t += nt) tile[t] = psi[base + offset(t)];
+  grid_wait();
+  for (uint32_t t = tid; t < T; t += nt) {
+    const C a = psi[base + offset(t)];
+    re[t] = a.x, im[t] = a.y;
+  }
   __syncthreads();
 
   R up = 0, dn = 0;
   for (int k = 0; k < d.nops; ++k) {
-    const Op op = ops[d.op0 + k];
+    const SOp op = s_ops[k];
     if (op.kind == OP_GATE) {
-      const GateCoef g = coefs[op.coef];
-      const R c1 = sizeof(R) == 8 ? (R)g.t : (R)g.tf;
-      const R s = sizeof(R) == 8 ? (R)g.s : (R)g.sft;
       const int lo = op.u < op.v ? op.u : op.v, hi = op.u < op.v ? op.v : op.u;
       const uint32_t bu = 1u << op.u, bv = 1u << op.v;
-      for (uint32_t p = tid; p < (T >> 2); p += nt) {
-        const uint32_t t0 = insert_zero(insert_zero(p, lo), hi);
-        C a = tile[t0 | bu], b = tile[t0 | bv];
-        shear_rotate(a, b, c1, s);
-        tile[t0 | bu] = a;
-        tile[t0 | bv] = b;
+      // task w: pair w mod T/4 and the plane (re a, im b) or (re b, im a)
+      for (uint32_t w = tid; w < (T >> 1); w += nt) {
+        const bool second = w >= (T >> 2);
+        const uint32_t t0 = insert_zero(insert_zero(second ? w - (T >> 2) : w, lo), hi);
+        R *const px = re + (t0 | (second ? bv : bu)), *const py = im + (t0 | (second ? bu : bv));
+        R x = *px, y = *py;
+        shear_plane(x, y, op.t, op.s);
+        *px = x, *py = y;
       }
       __syncthreads();
     } else if (op.kind == OP_DIAG) {
@@ -602,8 +632,10 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
           for (int b = a + 1; b < K; ++b)
             th += (ba ^ ((t >> b) & 1u)) ? (0ull - sQ[a * K + b]) : sQ[a * K + b];
         }
-        const C e = cis_turns(th, (R)0);
-        tile[t] = cmul(tile[t], e);
+        C a;
+        a.x = re[t], a.y = im[t];
+        a = cmul(a, cis_turns(th, (R)0));
+        re[t] = a.x, im[t] = a.y;
       }
       __syncthreads();
     } else if (op.kind == OP_REDUCE) {
@@ -611,8 +643,7 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
 #pragma unroll
       for (int q = 0; q < kMaxK; ++q) uhi[q] = 0;
       for (uint32_t t = tid; t < T; t += nt) {
-        const C a = tile[t];
-        const R pr = a.x * a.x + a.y * a.y;
+        const R pr = re[t] * re[t] + im[t] * im[t];
         const uint64_t bit = d.site_tile >= 0 ? ((t >> d.site_tile) & 1u)
                                               : ((base >> d.site_pos) & 1ull);
         if (bit) up += pr;
@@ -634,15 +665,16 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
       __syncthreads();  // later ops overwrite the tile
     }
   }
-  if (!d.relabel) {
-    for (uint32_t t = tid; t < T; t += nt) psi[base + offset(t)] = tile[t];
-  } else {
-    // output tile bit q holds the spin that input tile bit perm[q] held
-    for (uint32_t t = tid; t < T; t += nt) {
-      uint32_t ti = 0;
+  // output tile bit q holds the spin that input tile bit perm[q] held
+  for (uint32_t t = tid; t < T; t += nt) {
+    uint32_t ti = t;
+    if (d.relabel) {
+      ti = 0;
       for (int q = 0; q < K; ++q) ti |= ((t >> q) & 1u) << d.perm[q];
-      psi[base + offset(t)] = tile[ti];
     }
+    C a;
+    a.x = re[ti], a.y = im[ti];
+    psi[base + offset(t)] = a;
   }
   if constexpr (SITES)
     if (d.has_reduce) write_site_partials(d, M, base, s_w, jp.psites);
@@ -768,7 +800,7 @@ __device__ __forceinline__ void shear_lo_hi(u64 &P, u64 &Q, float t, float n) {
 }
 
 // Gate on register bits (JU + 1, JV + 1): two amplitude pairs per packed
-// instruction, same three-shear update as shear_rotate, in place.
+// instruction, same three-shear update as shear_plane, in place.
 template <int NP, int JU, int JV>
 __device__ __forceinline__ void gate_packed(u64 (&RE)[NP], u64 (&IM)[NP], float t, float s) {
   const u64 t2 = pack2(t, t), n2 = pack2(-s, -s);
@@ -1128,7 +1160,7 @@ __device__ __noinline__ void diag_tile(float2 *tile2, const uint64_t *__restrict
 // 2^JU ^ 2^JV), j with bit JU set, by P[j] += T P[k]; P[k] += S P[j]; P[j] +=
 // T P[k] (packed FP32x2), with T = (t, -t), S = (-s, s) when amplitude j is
 // stored (Re, Im) and both negated when it is stored (Im, Re): the three
-// shears of shear_rotate, the second plane's written y-first (y -= t x,
+// shears of shear_plane, the second plane's written y-first (y -= t x,
 // x += s y, y -= t x, the same rotation).  Orientation of j = parity of its
 // first-colour register bits (compile time) XOR the thread's (folded into T, S).
 // parity of the low nb bits of j (folded to a constant for a constant j)
@@ -1585,7 +1617,7 @@ template <int RB, bool SITES, bool ORIENT, bool DIRECT>
 __global__ void __launch_bounds__(RB == 5 ? 512 : 256)
 sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops1,
               const __grid_constant__ PassDesc d, const PhaseDesc *__restrict__ phases, int M,
-              unsigned ahead) {
+              unsigned ahead, bool chained) {
   // one job (gridDim.y == 1): its amplitude and op arrays come with the launch
   // so the tile copies can start at once; the rest of the job's pointers
   // (and everything for a batch) from the job table
@@ -1600,13 +1632,12 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   const int tid = threadIdx.x, nt = blockDim.x;
   const int lognt = d.K - RB;
   const uint64_t base = sw2::tile_origin(blockIdx.x, d, M);
-  // the tile's copies first, then the pass's program (coefficients already
-  // resolved for this dt), then the L2 prefetch of the tile of block
-  // blockIdx.x + ahead (ahead = blocks resident at once): DRAM keeps
-  // streaming while tiles compute, and that block's copies find its tile in L2
-  sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
-  if constexpr (DIRECT) sw2::load_direct<RB>(psi, base, d, tid, lognt, RE, IM);
-  else sw2::load_tile<RB>(psi, base, d, tid, lognt, (uint32_t)__cvta_generic_to_shared(tile2));
+  // the pass's program (coefficients already resolved for this dt) and, when
+  // chained, the outer fields while the sweep before this one finishes, then
+  // the tile, then the L2 prefetch of the tile of block blockIdx.x + ahead
+  // (ahead = blocks resident at once): DRAM keeps streaming while tiles
+  // compute, and that block's loads find its tile in L2
+  grid_go();
   {
     const uint32_t *pw = reinterpret_cast<const uint32_t *>(phases + d.phase0);
     const uint32_t a_ph = (uint32_t)__cvta_generic_to_shared(s_ph);
@@ -1616,9 +1647,14 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
     const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
     for (int i = tid; i < d.nrops; i += nt) sw2::cp_async16(a_op + 16u * i, so + i);
   }
+  if (chained && d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
+  grid_wait();
+  sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
+  if constexpr (DIRECT) sw2::load_direct<RB>(psi, base, d, tid, lognt, RE, IM);
+  else sw2::load_tile<RB>(psi, base, d, tid, lognt, (uint32_t)__cvta_generic_to_shared(tile2));
   if (ahead && blockIdx.x + ahead < gridDim.x)
     sw2::prefetch_tile<RB>(psi, sw2::tile_origin(blockIdx.x + ahead, d, M), d, tid, lognt);
-  if (d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
+  if (!chained && d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   sw2::cp_async_wait_all();
   __syncthreads();
 

@@ -15,7 +15,7 @@ namespace spinrp {
 // shared memory as 16-byte amplitudes with a three-bit XOR swizzle (sw2d::slot),
 // so one 16-byte access moves one amplitude and the eight lanes of an access
 // quarter (three lane bits of distinct residues mod 3) hit distinct 16-byte
-// bank groups.  Gates are the same three shears per plane as shear_rotate.
+// bank groups.  Gates are the same three shears per plane as shear_plane.
 // ===========================================================================
 namespace sw2d {
 
@@ -84,6 +84,21 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
   const int lognt = K - RB;
   const uint64_t base = sw2::tile_origin(blockIdx.x, d, M);
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(tile16);
+  grid_go();
+  // the pass's program; FP64 coefficients from the job's table
+  for (int i = tid; i < d.nphases; i += nt) s_ph[i] = phases[d.phase0 + i];
+  for (int i = tid; i < d.nrops; i += nt) {
+    const ROp r = rops[d.rop0 + i];
+    sw2d::SOpD o;
+    o.kind = r.kind, o.combo = r.combo, o.arg = r.arg;
+    o.t = 0.0, o.s = 0.0;
+    if (r.kind == OP_GATE) {
+      const GateCoef g = jp.coefs[r.coef];
+      o.t = g.t, o.s = g.s;
+    }
+    s_op[i] = o;
+  }
+  grid_wait();
   // ---- global -> shared: 16-byte async copies, amplitude a = tid + nt * e,
   // e in Gray-code order in runs of eight (as in the complex64 kernel)
   {
@@ -115,19 +130,6 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
       }
       sw2::cp_async16(sbase + sb, src);
     }
-  }
-  // the pass's program; FP64 coefficients from the job's table
-  for (int i = tid; i < d.nphases; i += nt) s_ph[i] = phases[d.phase0 + i];
-  for (int i = tid; i < d.nrops; i += nt) {
-    const ROp r = rops[d.rop0 + i];
-    sw2d::SOpD o;
-    o.kind = r.kind, o.combo = r.combo, o.arg = r.arg;
-    o.t = 0.0, o.s = 0.0;
-    if (r.kind == OP_GATE) {
-      const GateCoef g = jp.coefs[r.coef];
-      o.t = g.t, o.s = g.s;
-    }
-    s_op[i] = o;
   }
   // L2 prefetch of the tile of block blockIdx.x + ahead (128-byte runs: tile
   // bits 0..2, the low physical bits)
