@@ -714,9 +714,14 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
       std::vector<ROp> pending;  // element-wise ops waiting for the next phase
       d.direct = want_direct;
       // lanes: bits that should be lane bits if they are not in registers
-      auto new_phase = [&](const std::vector<int> &rb, const std::vector<int> &prefer = {}) {
+      auto new_phase = [&](std::vector<int> rb, const std::vector<int> &prefer = {}) {
         PhaseDesc ph;
         memset(&ph, 0, sizeof ph);
+        // a readout without gates: its spin on the last register bit
+        for (const ROp &r : pending)
+          if (rounds && r.kind == OP_REDUCE)
+            for (int k = 0; k < RB; ++k)
+              if (rb[k] == d.site_tile) std::swap(rb[k], rb[RB - 1]);
         uint32_t isreg = 0;
         for (int k = 0; k < RB; ++k) ph.rb[k] = (uint8_t)rb[k], isreg |= 1u << rb[k];
         // lane bits: nres non-register bits of distinct residues mod nres
@@ -808,8 +813,11 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
               if ((sets[k] >> q) & 1) rb.push_back(q);
             std::vector<PhaseRound> rounds_of;
             const bool first = first_of && k == 0, last = last_of && k + 1 == sets.size();
-            plan_rounds(pg, RB, split, last ? d.perm[0] : first ? 0 : -1, last ? d.perm[1] : first ? 1 : -1, &rb,
-                        &rounds_of);
+            const int fix1 = last ? d.perm[0] : first ? 0 : -1, fix2 = last ? d.perm[1] : first ? 1 : -1;
+            // the readout spin on the last register bit, unless it is a fixed one
+            const bool hold = split >= 0 && d.site_tile >= 0 && ((sets[k] >> d.site_tile) & 1) &&
+                              d.site_tile != fix1 && d.site_tile != fix2;
+            plan_rounds(pg, RB, split, fix1, fix2, hold ? d.site_tile : -1, &rb, &rounds_of);
             if (last) new_phase(rb, {d.perm[2], d.perm[3]});
             else new_phase(rb);
             for (const PhaseRound &rd : rounds_of) {
@@ -937,6 +945,35 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
         ps->phases.insert(ps->phases.end(), phases.begin(), phases.end());
         ps->rops.resize(d.rop0);
         ps->rops.insert(ps->rops.end(), rops.begin(), rops.end());
+      }
+    }
+    // a plain complex64 pass's steps, and where its readout's phase has spin 1
+    d.site_label = d.site_thr = -1;
+    if (rounds) {
+      int ns = 0;
+      for (int p = d.phase0; p < (int)ps->phases.size(); ++p) {
+        const PhaseDesc &ph = ps->phases[p];
+        std::vector<uint32_t> st;
+        for (int k = 0; k < ph.nops; ++k) {
+          const ROp &r = ps->rops[ph.op0 + k];
+          if (r.kind == OP_ROUND) st.push_back((uint32_t)r.coef | (uint32_t)r.arg << 16), k += r.arg;
+          else st.push_back(r.kind == OP_REDUCE ? kStepReduce : kStepDiag);
+          if (r.kind != OP_REDUCE || d.site_tile < 0) continue;
+          for (int i = 0; i < RB; ++i)
+            if (ph.rb[i] == d.site_tile) d.site_label = i;
+          for (int i = 0; i < K - RB; ++i)
+            if ((i < 5 ? ph.lanes[i] : ph.warps[i - 5]) == d.site_tile) d.site_thr = i;
+          if (d.site_label < 0 ? d.site_thr < 0 : d.site_label > 2 && d.site_label != RB - 1) {
+            *err = "readout spin out of place";
+            return false;
+          }
+        }
+        if (st.empty()) st.push_back(0u);
+        if (ns + (int)st.size() > kMaxPassSteps) {
+          *err = "a sweep has too many steps";
+          return false;
+        }
+        for (size_t k = 0; k < st.size(); ++k) d.steps[ns++] = st[k] | (k + 1 == st.size() ? kStepEnd : 0u);
       }
     }
     // the diagonal op's tables (the same tile bits in every pass that has one)
@@ -1524,7 +1561,7 @@ static size_t resident_bytes(const Plan &plan, const PassSet &ps, int prec, bool
   if (ps.only < 0 || ps.first < 0 || ps.midstep < 0 || ps.last < 0) return 0;
   if (plan.M - ps.rb > 8) return 0;  // at most 256 threads per block
   const size_t b = (size_t(8) << plan.M) + sizeof(PhaseDesc) * ps.phases.size() +
-                   sizeof(ROpRes) * (ps.rops.size() + 1);  // a round reads one coefficient ahead
+                   sizeof(ROpRes) * (ps.rops.size() + 2);  // coefficients are read ahead
   return b <= kResidentMaxSmem ? b : 0;
 }
 
@@ -2502,8 +2539,32 @@ extern "C" int spinrp_system_plan_check(const spinrp_system *sys, int prec, doub
       for (int a = 0; a < ps.rb; ++a)
         for (int bb = a + 1; bb < ps.rb; ++bb) KU.push_back(a), KV.push_back(bb);
     }
+    int ns = 0;
     for (int p = 0; p < d.nphases; ++p) {
       const PhaseDesc &ph = ps.phases[d.phase0 + p];
+      if (prec == SPINRP_C64 && !ps.oriented) {
+        // the phase's steps, walked as the kernel walks them, are its ops
+        int k = 0;
+        for (bool end = false; !end; ++ns) {
+          if (ns >= kMaxPassSteps) return fail(SPINRP_EINVAL, "plan_check: pass %zu: steps", pi);
+          const uint32_t w = d.steps[ns];
+          end = (w & kStepEnd) != 0;
+          if (ph.nops == 0 && end && w == kStepEnd) continue;
+          const ROp &r = ps.rops[ph.op0 + std::min(k, ph.nops - 1)];
+          const bool ok = k < ph.nops && ((w & kStepReduce) ? r.kind == OP_REDUCE
+                                          : (w & kStepDiag) ? r.kind == OP_DIAG && ph.nops == 1
+                                                            : r.kind == OP_ROUND && (w & 0x7fffu) == (uint32_t)r.coef &&
+                                                                  ((w >> 16) & 0xffu) == r.arg);
+          if (!ok) return fail(SPINRP_EINVAL, "plan_check: pass %zu phase %d: steps", pi, p);
+          k += r.kind == OP_ROUND ? 1 + r.arg : 1;
+        }
+        if (k != ph.nops) return fail(SPINRP_EINVAL, "plan_check: pass %zu phase %d: steps end early", pi, p);
+        for (int i = 0; i < ph.nops; ++i)
+          if (ps.rops[ph.op0 + i].kind == OP_REDUCE && d.site_tile >= 0 &&
+              (d.site_label >= 0 ? ph.rb[d.site_label] : d.site_thr < 5 ? ph.lanes[d.site_thr]
+                                                                        : ph.warps[d.site_thr - 5]) != d.site_tile)
+            return fail(SPINRP_EINVAL, "plan_check: pass %zu phase %d: readout spin", pi, p);
+      }
       uint32_t seen = 0;
       for (int k = 0; k < ps.rb; ++k) seen |= 1u << ph.rb[k];
       for (int k = 0; k < 5; ++k) seen |= 1u << ph.lanes[k];

@@ -19,6 +19,13 @@ enum OpKind : uint8_t {
   OP_ROUND = 4,   // register-blocked plain complex64 programs: heads a round of gates (see ROp)
 };
 
+// Steps of a plain complex64 pass's phases, in order: a round (its pairs in bits
+// 0..14, its number of gates in bits 16..23), the readout or the diagonal op;
+// the last of a phase has kStepEnd.  They come with the pass descriptor, a
+// kernel parameter, so the kernels branch on them uniformly.
+constexpr int kMaxPassSteps = 160;
+constexpr uint32_t kStepEnd = 1u << 31, kStepReduce = 1u << 30, kStepDiag = 1u << 29;
+
 // One operation of a sweep, in tile-local bit indices.
 struct Op {
   uint8_t kind;
@@ -61,6 +68,11 @@ struct PassDesc {
   // positions that hold spins of the first colour, input layout
   uint32_t black_tile;
   uint64_t black_outer;
+  // plain complex64 programs: register bit of the readout spin in the readout's
+  // phase (-1: not one; 0, 1, 2 or the last), else its thread-index bit (-1: an
+  // outer bit); the phases' steps
+  int32_t site_label, site_thr;
+  uint32_t steps[kMaxPassSteps];
 };
 
 // Register-blocked execution of a pass.  In a phase every thread holds the
@@ -69,17 +81,17 @@ struct PassDesc {
 // the phase's ops to them in registers and writes them back to shared memory.
 // lanes[]/warps[] give the tile bits the thread index supplies.
 constexpr int kMaxRegBits = 6;  // 5 or 6 register bits per phase
-struct PhaseDesc {
+struct alignas(16) PhaseDesc {
+  uint16_t tslot[kMaxK - 4]; // slot of each thread-index bit (lanes, then warps; unused ones zero)
+  uint16_t sm[kMaxRegBits];  // shared-memory slot of each register bit
+  int32_t op0;
   uint8_t rb[kMaxRegBits];
   uint8_t lanes[5];
   uint8_t warps[kMaxK - 10];
   uint8_t nops;
   uint8_t nb;  // oriented program: register bits 0..nb-1 hold first-colour spins
-  int32_t op0;
-  uint16_t sm[kMaxRegBits];  // shared-memory slot of each register bit
-  uint16_t tslot[kMaxK - 5]; // slot of each thread-index bit (lanes, then warps)
-  uint16_t pad2;
 };
+static_assert(kMaxK == 14 && kMaxRegBits == 6, "the kernels read tslot and sm as two 16-byte words");
 
 // A pass's register-blocked program is staged in shared memory; passes with
 // more phases or ops than this run the plain sweep kernel instead.
@@ -145,7 +157,7 @@ struct ROpRes {
   uint32_t tab;  // diagonal op: offset of its variant's table (8-byte words)
 };
 static_assert(sizeof(ROpRes) == 16, "ROpRes is copied in 16-byte pieces");
-static_assert(sizeof(PhaseDesc) % 4 == 0, "PhaseDesc is copied in 4-byte pieces");
+static_assert(sizeof(PhaseDesc) % 16 == 0, "PhaseDesc is copied in 16-byte pieces");
 
 // Device pointers of one job (one state) as the kernels see them; a launch
 // covers gridDim.y jobs that share one sweep plan, block row y using jobs[y].
@@ -227,12 +239,12 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
 // scalar) and cuts the gates into rounds, walks over the register-bit pairs in
 // lexicographic order that keep every bit's gate sequence, for few rounds and few gates on the pack bit.  An empty round
 // stands for the readout after the first `split` gates (split < 0: none).
-// fix1, fix2: tile bits that register bits 1 and 2 hold (-1: any).
+// fix1, fix2, fix_last: tile bits that register bits 1, 2 and RB - 1 hold (-1: any).
 struct PhaseRound {
   std::vector<int> gates;  // indices into the phase's gates, in execution order
   std::vector<int> combo;  // register-bit pair of every gate of the phase
 };
 void plan_rounds(const std::vector<std::pair<int, int>> &gates, int RB, int split, int fix1, int fix2,
-                 std::vector<int> *rb, std::vector<PhaseRound> *rounds);
+                 int fix_last, std::vector<int> *rb, std::vector<PhaseRound> *rounds);
 
 }  // namespace spinrp

@@ -1428,22 +1428,37 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
                                            u64 (&RE)[1 << (RB - 1)], u64 (&IM)[1 << (RB - 1)], float2 *psi) {
   constexpr int NP = 1 << (RB - 1);
   const uint32_t outer_par = ORIENT ? (uint32_t)(__popcll(base & d.black_outer) & 1) : 0u;
+  // masks of the thread-index bits, two to a word
+  uint32_t tm[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i)
+    tm[i] = (((tid >> (2 * i)) & 1) ? 0xffffu : 0u) | (((tid >> (2 * i + 1)) & 1) ? 0xffff0000u : 0u);
+  int st = 0;  // step of the pass
   for (int p = 0; p < d.nphases; ++p) {
     const PhaseDesc &ph = s_ph[p];
     // slot of this thread's subcube origin (host-precomputed slot of each
-    // thread-index bit) and of the register bits
-    uint32_t s0 = 0;
-    for (int b = 0; b < lognt; ++b)
-      if ((tid >> b) & 1) s0 ^= ph.tslot[b];
+    // thread-index bit) and of the register bits, from two 16-byte words (bit
+    // by bit these loads took 430 cycles a phase)
+    const uint4 w0 = reinterpret_cast<const uint4 *>(&ph)[0], w1 = reinterpret_cast<const uint4 *>(&ph)[1];
+    const uint32_t sx = (w0.x & tm[0]) ^ (w0.y & tm[1]) ^ (w0.z & tm[2]) ^ (w0.w & tm[3]) ^ (w1.x & tm[4]);
+    const uint32_t s0 = (sx ^ (sx >> 16)) & 0xffffu;
     uint32_t sm[RB];
 #pragma unroll
-    for (int k = 0; k < RB; ++k) sm[k] = ph.sm[k];
+    for (int k = 0; k < RB; ++k) {
+      const uint32_t v = k < 2 ? w1.y : k < 4 ? w1.z : w1.w;
+      sm[k] = (k & 1) ? v >> 16 : v & 0xffffu;
+    }
     const int o0 = ph.op0 - d.rop0;
-    if (DIAG && ph.nops == 1 && s_op[o0].kind == OP_DIAG) {
+    // the phase's first step, and the coefficients of its first gate if it is a round
+    uint32_t step = ORIENT ? 0u : d.steps[st];
+    if (DIAG && (ORIENT ? ph.nops == 1 && s_op[o0].kind == OP_DIAG : (step & kStepDiag) != 0)) {
       diag_tile<RB, ORIENT>(tile2, dtab + s_op[o0].tab, sH, d.K, tid, lognt, d.black_tile, outer_par);
       sync();
+      ++st;
       continue;
     }
+    float2 ts = make_float2(0.f, 0.f);
+    if constexpr (WALK && !ORIENT) ts = make_float2(s_op[o0 + 1].t, s_op[o0 + 1].s);
     if constexpr (ORIENT) {
       oriented_phase<RB, SITES>(tile2, d, ph, s_op + o0, base, tid, lognt, up, dn, s_w, s0, sm, outer_par);
       sync();
@@ -1476,40 +1491,40 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
         IM[j] = pack2(v0.y, v1.y);
       }
     }
-    for (int k = 0; k < ph.nops; ++k) {
-      const ROpRes cur = s_op[o0 + k];
-      if (!WALK && cur.kind == OP_GATE) {
-        gate_combo(RE, IM, cur.combo, cur.t, cur.s);
-      } else if (WALK && cur.kind == OP_ROUND) {
-        const ROpRes *first = s_op + o0 + k + 1;
-        const float2 ts = make_float2(first->t, first->s);
-        run_round<NP>(RE, IM, cur.tab, first, ts);
-        k += cur.arg;
-      } else if (cur.kind == OP_REDUCE) {
-        int kr = -1;
-#pragma unroll
-        for (int q = 0; q < RB; ++q)
-          if (ph.rb[q] == d.site_tile) kr = q;
-        uint32_t fixed_bit;
-        if (d.site_tile < 0) {
-          fixed_bit = (uint32_t)((base >> d.site_pos) & 1ull);
+    for (int k = o0;;) {  // op of the step
+      if ((step & kStepReduce) == 0) {
+        const int n = (int)(step >> 16) & 0xff;
+        if constexpr (WALK) {
+          run_round<NP>(RE, IM, step & 0x7fffu, s_op + k + 1, ts);
         } else {
-          uint32_t t0 = 0;
-          for (int b = 0; b < 5; ++b) t0 |= ((uint32_t)(tid >> b) & 1u) << ph.lanes[b];
-          for (int b = 0; b < lognt - 5; ++b) t0 |= ((uint32_t)(tid >> (5 + b)) & 1u) << ph.warps[b];
-          fixed_bit = (t0 >> d.site_tile) & 1u;
+          for (int i = 1; i <= n; ++i) {
+            const ROpRes cur = s_op[k + i];
+            gate_combo(RE, IM, cur.combo, cur.t, cur.s);
+          }
         }
+        k += 1 + n;
+      } else {
+        // weights by register bits 1, 2 and RB - 1 (and the pack bit, the lanes),
+        // one of which the readout spin is if it is a register bit at all (with
+        // the spin's register bit found at run time and every pack tested for
+        // it, this took 1300 cycles of a lone warp)
+        u64 acc[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) acc[i] = 0ull;
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
-          const float2 pr = unpack2(fma2(RE[j], RE[j], mul2(IM[j], IM[j])));
-          if (kr == 0) {
-            dn += pr.x;
-            up += pr.y;
-          } else {
-            const uint32_t bit = kr > 0 ? ((uint32_t)(j >> (kr - 1)) & 1u) : fixed_bit;
-            if (bit) up += pr.x + pr.y;
-            else dn += pr.x + pr.y;
-          }
+          u64 &a = acc[(j & 3) | ((j >> (RB - 2)) << 2)];
+          a = add2(a, fma2(RE[j], RE[j], mul2(IM[j], IM[j])));
+        }
+        const int L = d.site_label;
+        const uint32_t bit = d.site_thr >= 0 ? (uint32_t)(tid >> d.site_thr) & 1u
+                                             : (uint32_t)((base >> d.site_pos) & 1ull);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float2 v = unpack2(acc[i]);
+          const bool hi = L == 1 ? (i & 1) != 0 : L == 2 ? (i & 2) != 0 : L > 2 ? (i & 4) != 0 : bit != 0;
+          up += L == 0 ? v.y : hi ? v.x + v.y : 0.f;
+          dn += L == 0 ? v.x : hi ? 0.f : v.x + v.y;
         }
         if constexpr (SITES) {
           // per tile bit, the weight with that bit up: register bits from the
@@ -1540,7 +1555,12 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
           }
           warp_site_sum<float>(tsum, kMaxK, s_w);
         }
+        ++k;
       }
+      ++st;
+      if (step & kStepEnd) break;
+      step = d.steps[st];
+      if constexpr (WALK) ts = make_float2(s_op[k + 1].t, s_op[k + 1].s);
     }
     if (ENDS == kDirect && p == d.nphases - 1) {
       // one phase only: every load of the tile before its relabelled stores
@@ -1639,7 +1659,7 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   extern __shared__ __align__(16) float2 tile2[];
   __shared__ uint64_t sH[kMaxK + 1];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
-  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 1];  // a round reads one coefficient ahead
+  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 2];  // coefficients are read ahead
   __shared__ double s_w[SITES ? kMaxWarps * kSiteSlots : 1];
   const int tid = threadIdx.x, nt = blockDim.x;
   const int lognt = d.K - RB;
@@ -1651,10 +1671,10 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   // compute, and that block's loads find its tile in L2
   grid_go();
   {
-    const uint32_t *pw = reinterpret_cast<const uint32_t *>(phases + d.phase0);
+    const char *pw = reinterpret_cast<const char *>(phases + d.phase0);
     const uint32_t a_ph = (uint32_t)__cvta_generic_to_shared(s_ph);
-    const int nw = d.nphases * (int)(sizeof(PhaseDesc) / 4);
-    for (int i = tid; i < nw; i += nt) sw2::cp_async4(a_ph + 4u * i, pw + i);
+    const int nw = d.nphases * (int)(sizeof(PhaseDesc) / 16);
+    for (int i = tid; i < nw; i += nt) sw2::cp_async16(a_ph + 16u * i, pw + 16 * i);
     const ROpRes *so = (one ? sops1 : jp.sops) + d.rop0;
     const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
     for (int i = tid; i < d.nrops; i += nt) sw2::cp_async16(a_op + 16u * i, so + i);
@@ -1711,10 +1731,10 @@ resident_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ Reside
   // the state (tile bits = physical bits: base 0, no relabelling), then the program
   sw2::load_tile<RB>(psi, 0, rp.first, tid, lognt, (uint32_t)__cvta_generic_to_shared(tile2));
   {
-    const uint32_t *pw = reinterpret_cast<const uint32_t *>(phases);
+    const char *pw = reinterpret_cast<const char *>(phases);
     const uint32_t a_ph = (uint32_t)__cvta_generic_to_shared(s_ph);
-    const int nw = nph * (int)(sizeof(PhaseDesc) / 4);
-    for (int i = tid; i < nw; i += nt) sw2::cp_async4(a_ph + 4u * i, pw + i);
+    const int nw = nph * (int)(sizeof(PhaseDesc) / 16);
+    for (int i = tid; i < nw; i += nt) sw2::cp_async16(a_ph + 16u * i, pw + 16 * i);
     const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
     for (int i = tid; i < nrops; i += nt) sw2::cp_async16(a_op + 16u * i, jp.sops + i);
   }

@@ -179,7 +179,7 @@ persist_kernel(const PersistPlan *__restrict__ plan, unsigned long long *queue, 
   extern __shared__ __align__(16) float2 tile2[];
   __shared__ uint64_t sH[kMaxK + 1];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
-  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 1];  // a round reads one coefficient ahead
+  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 2];  // coefficients are read ahead
   __shared__ __align__(16) PassDesc s_d;
   __shared__ double s_up[8], s_dn[8];
   __shared__ unsigned long long s_item;
@@ -260,10 +260,10 @@ persist_kernel(const PersistPlan *__restrict__ plan, unsigned long long *queue, 
     const int lognt = d.K - RB, M = G.M;
     const uint64_t base = sw2::tile_origin(r, d, M);
     {
-      const uint32_t *pw = reinterpret_cast<const uint32_t *>(G.phases + d.phase0);
+      const char *pw = reinterpret_cast<const char *>(G.phases + d.phase0);
       const uint32_t a_ph = (uint32_t)__cvta_generic_to_shared(s_ph);
-      const int nw = d.nphases * (int)(sizeof(PhaseDesc) / 4);
-      for (int q = tid; q < nw; q += nt) sw2::cp_async4(a_ph + 4u * q, pw + q);
+      const int nw = d.nphases * (int)(sizeof(PhaseDesc) / 16);
+      for (int q = tid; q < nw; q += nt) sw2::cp_async16(a_ph + 16u * q, pw + 16 * q);
       const ROpRes *so = jp.sops + d.rop0;
       const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
       for (int q = tid; q < d.nrops; q += nt) sw2::cp_async16(a_op + 16u * q, so + q);

@@ -195,7 +195,7 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
   __shared__ uint64_t sH[2][kMaxK + 1];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
   // one job: the pass's ops; BATCH: three slices of kPipeBatchOps, one per buffer
-  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 1];  // a round reads one coefficient ahead
+  __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 2];  // coefficients are read ahead
   __shared__ __align__(16) JobPtrs s_job[BATCH ? 3 : 1];
   __shared__ __align__(8) uint64_t s_full[3], s_done[3];
   __shared__ double s_up[2][NW], s_dn[2][NW];
@@ -215,10 +215,10 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
 
   // the pass's program, once for the whole sweep (one job: its ops too)
   {
-    const uint32_t *pw = reinterpret_cast<const uint32_t *>(phases + d.phase0);
+    const char *pw = reinterpret_cast<const char *>(phases + d.phase0);
     const uint32_t a_ph = (uint32_t)__cvta_generic_to_shared(s_ph);
-    const int nw = d.nphases * (int)(sizeof(PhaseDesc) / 4);
-    for (int i = tid; i < nw; i += kPipeThreads) sw2::cp_async4(a_ph + 4u * i, pw + i);
+    const int nw = d.nphases * (int)(sizeof(PhaseDesc) / 16);
+    for (int i = tid; i < nw; i += kPipeThreads) sw2::cp_async16(a_ph + 16u * i, pw + 16 * i);
     if (!BATCH) {
       const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
       for (int i = tid; i < d.nrops; i += kPipeThreads) sw2::cp_async16(a_op + 16u * i, sops1 + d.rop0 + i);

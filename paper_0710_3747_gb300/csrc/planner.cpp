@@ -464,7 +464,7 @@ int greedy_rounds(const std::vector<int> &ku, const std::vector<int> &kv, const 
 }  // namespace
 
 void plan_rounds(const std::vector<std::pair<int, int>> &gates, int RB, int split, int fix1, int fix2,
-                 std::vector<int> *rb, std::vector<PhaseRound> *rounds) {
+                 int fix_last, std::vector<int> *rb, std::vector<PhaseRound> *rounds) {
   const int n = (int)gates.size();
   std::vector<int> order = *rb, best_order;  // order[k]: tile bit of register bit k
   std::sort(order.begin(), order.end());
@@ -484,7 +484,9 @@ void plan_rounds(const std::vector<std::pair<int, int>> &gates, int RB, int spli
   // a gate on the pack bit costs a gate more, a round about two (its tests)
   int best = std::numeric_limits<int>::max();
   do {
-    if ((fix1 >= 0 && order[1] != fix1) || (fix2 >= 0 && order[2] != fix2)) continue;
+    if ((fix1 >= 0 && order[1] != fix1) || (fix2 >= 0 && order[2] != fix2) ||
+        (fix_last >= 0 && order[RB - 1] != fix_last))
+      continue;
     const int pack = label();
     if (pack >= best) continue;
     const int r = greedy_rounds(ku, kv, combo, RB, 0, cut, nullptr) + greedy_rounds(ku, kv, combo, RB, cut, n, nullptr);
