@@ -395,9 +395,9 @@ struct PassSet {
   DiagTab tab;            // tables of the diagonal op
   // pipe_kernel's variant for a pass: with the diagonal op; else by its gates
   // per phase (a walk over the register-bit pairs pays from kPipeDenseGates on)
-  int variant(int pass) const {
+  int variant(int pass, bool sites) const {
     const PassDesc &d = desc[pass];
-    return d.diag >= 0 ? kPipeDiag : d.nops >= kPipeDenseGates * d.nphases ? kPipeDense : kPipeSparse;
+    return sites ? kPipeSites : d.diag >= 0 ? kPipeDiag : d.nops >= kPipeDenseGates * d.nphases ? kPipeDense : kPipeSparse;
   }
 };
 
@@ -1142,6 +1142,7 @@ static int set_smem_limits() {
     PIPE_SMEM(kPipeSparse);
     PIPE_SMEM(kPipeDense);
     PIPE_SMEM(kPipeDiag);
+    CUDA_TRY(cudaFuncSetAttribute(pipe_kernel<6, 13, false, kPipeSites>, a, (int)kPipeSmem));
 #undef PIPE_SMEM
     CUDA_TRY(cudaFuncSetAttribute(resident_kernel<5, false>, a, (int)kResidentMaxSmem));
     CUDA_TRY(cudaFuncSetAttribute(resident_kernel<5, true>, a, (int)kResidentMaxSmem));
@@ -1640,7 +1641,7 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
     const unsigned ahead = c.prefetch_ahead;
     const ROpRes *sops1 = c.njobs == 1 ? c.job0.sops : nullptr;
     const int code = (c.rb == 6 ? 4 : 0) | (sites ? 2 : 0) | (c.oriented ? 1 : 0);
-    const bool piped = c.pipe_blocks && K == 13 && code == 4;
+    const bool piped = c.pipe_blocks && K == 13 && (code & ~2) == 4 && !(sites && c.njobs > 1);
     if (piped) {
 #define PIPE(B_, V_)                                                                                             \
   CUDA_TRY(launch_sweep(chained, dim3(c.pipe_blocks), kPipeThreads, kPipeSmem, stream, pipe_kernel<6, 13, B_, V_>, \
@@ -1648,13 +1649,14 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
                         B_ ? c.job_stride : 0ll, pd, c.phases, c.M, c.pipe_err, 0))
       const JobPtrs &j0 = c.njobs == 1 ? c.job0 : c.batch0;
       const bool many = c.njobs > 1;
-      switch (2 * c.ps->variant(pass) + (many ? 1 : 0)) {
+      switch (2 * c.ps->variant(pass, sites) + (many ? 1 : 0)) {
         case 2 * kPipeSparse: PIPE(false, kPipeSparse); break;
         case 2 * kPipeSparse + 1: PIPE(true, kPipeSparse); break;
         case 2 * kPipeDense: PIPE(false, kPipeDense); break;
         case 2 * kPipeDense + 1: PIPE(true, kPipeDense); break;
         case 2 * kPipeDiag: PIPE(false, kPipeDiag); break;
-        default: PIPE(true, kPipeDiag); break;
+        case 2 * kPipeDiag + 1: PIPE(true, kPipeDiag); break;
+        default: PIPE(false, kPipeSites); break;  // states only
       }
 #undef PIPE
       if (many && pd.has_reduce) {

@@ -154,35 +154,33 @@ __device__ void reduce_finalize(double up, double dn, const JobPtrs &jp, bool re
 constexpr int kSiteSlots = kMaxK + 1;  // tile bits 0..kMaxK-1, slot kMaxK = norm
 constexpr int kMaxWarps = 16;
 
-// Warp-sum v (in the thread's precision) and park it at s_w[warp][slot].
+// Warp-sum v (in the thread's precision) and park it at s_w[warp][slot]; tid:
+// the thread's index in the group that owns the tile.
 template <typename R>
-__device__ __forceinline__ void warp_site_sum(R v, int slot, double *s_w) {
+__device__ __forceinline__ void warp_site_sum(R v, int slot, double *s_w, int tid) {
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) s_w[(threadIdx.x >> 5) * kSiteSlots + slot] = (double)v;
+  if ((tid & 31) == 0) s_w[(tid >> 5) * kSiteSlots + slot] = (double)v;
 }
 
-// After a __syncthreads that follows every warp_site_sum: block sums over the
-// warps in order, written as this block's row of the (M + 1) columns.
-__device__ void write_site_partials(const PassDesc d, int M, uint64_t base, const double *s_w,
-                                    double *psites) {
-  const int nw = (blockDim.x + 31) >> 5, K = d.K;
-  const size_t nblk = gridDim.x, blk = blockIdx.x;
-  for (int i = threadIdx.x; i <= M; i += blockDim.x) {
-    double norm = 0.0;
-    for (int w = 0; w < nw; ++w) norm += s_w[w * kSiteSlots + kMaxK];
-    double v;
-    int col;
+// After a barrier that follows every warp_site_sum: sums over the warps of the
+// tile's nt threads in order, written as tile blk's row (of nblk) of the (M + 1)
+// columns.
+__device__ __forceinline__ void write_site_partials(const PassDesc &d, int M, uint64_t base, const double *s_w,
+                                                    double *psites, int tid, int nt, size_t blk, size_t nblk) {
+  const int nw = (nt + 31) >> 5, K = d.K;
+  for (int i = tid; i <= M; i += nt) {
+    // a tile bit's weight, or the tile's for an outer spin and the norm (one
+    // FP64 sum a thread: they run at 1/64 of the FP32 rate)
+    const int from = i < K ? i : kMaxK;
+    double v = 0.0;
+    for (int w = 0; w < nw; ++w) v += s_w[w * kSiteSlots + from];
+    int col = 0;
     if (i < K) {
-      v = 0.0;
-      for (int w = 0; w < nw; ++w) v += s_w[w * kSiteSlots + i];
       col = 1 + d.tile_spin[i];
     } else if (i < M) {
       const int o = i - K;
-      v = ((base >> d.outer_pos[o]) & 1ull) ? norm : 0.0;
+      if (!((base >> d.outer_pos[o]) & 1ull)) v = 0.0;
       col = 1 + d.outer_spin[o];
-    } else {
-      v = norm;
-      col = 0;
     }
     psites[col * nblk + blk] = v;
   }
@@ -659,8 +657,8 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
         // tile bits below L come from the thread index: the thread's whole sum
 #pragma unroll
         for (int q = 0; q < kMaxK; ++q)
-          warp_site_sum<R>(q < L ? (((tid >> q) & 1) ? tsum : (R)0) : uhi[q], q, s_w);
-        warp_site_sum<R>(tsum, kMaxK, s_w);
+          warp_site_sum<R>(q < L ? (((tid >> q) & 1) ? tsum : (R)0) : uhi[q], q, s_w, tid);
+        warp_site_sum<R>(tsum, kMaxK, s_w, tid);
       }
       __syncthreads();  // later ops overwrite the tile
     }
@@ -677,7 +675,7 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
     psi[base + offset(t)] = a;
   }
   if constexpr (SITES)
-    if (d.has_reduce) write_site_partials(d, M, base, s_w, jp.psites);
+    if (d.has_reduce) write_site_partials(d, M, base, s_w, jp.psites, tid, nt, blockIdx.x, gridDim.x);
   if (d.has_reduce) reduce_finalize((double)up, (double)dn, jp, false);
 }
 
@@ -1316,9 +1314,9 @@ __device__ __forceinline__ void oriented_phase(float2 *tile2, const PassDesc &d,
 #pragma unroll
           for (int k2 = 0; k2 < RB; ++k2)
             if (ph.rb[k2] == q) v = ureg[k2];
-          warp_site_sum<float>(v, q, s_w);
+          warp_site_sum<float>(v, q, s_w, tid);
         }
-        warp_site_sum<float>(tsum, kMaxK, s_w);
+        warp_site_sum<float>(tsum, kMaxK, s_w, tid);
       }
     }
     cur = nxt;
@@ -1409,6 +1407,70 @@ __device__ __forceinline__ void store_direct(float2 *psi, uint64_t base, const P
     asm volatile("st.global.v4.b64 [%0], {%1, %2, %3, %4};" ::"l"(dst), "l"(v[0]), "l"(v[1]), "l"(v[2]), "l"(v[3])
                  : "memory");
   }
+}
+
+// All-site readout of a phase: every tile bit's weight over the warp into
+// s_w[warp][bit] and the whole weight into slot kMaxK, from the thread's sums
+// acc (by register bits 1, 2, RB - 1 and the pack bit, in the lanes) and ext (by
+// the register bits between).  The register bits' sums are reduced together,
+// half of them exchanged at each step (9 shuffles for all), the lane bits'
+// build up along one butterfly (15), a warp bit's is the warp's whole sum or
+// nothing.  (A butterfly for each tile bit, 75 shuffles, its values picked from
+// the registers at run time, cost 30 us of an 84 us sweep of 2^23 amplitudes.)
+template <int RB>
+__device__ __forceinline__ void site_sums(const u64 (&acc)[8], const u64 (&ext)[2], const PhaseDesc &ph, int tid,
+                                          int lognt, double *s_w) {
+  const int lane = tid & 31, warp = tid >> 5;
+  double *const row = s_w + warp * kSiteSlots;
+  float v[8], T = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = 0.f;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const float2 x = unpack2(acc[i]);
+    const float y = x.x + x.y;
+    T += y, v[0] += x.y;
+    if (i & 1) v[1] += y;
+    if (i & 2) v[2] += y;
+    if (i & 4) v[RB - 1] += y;
+  }
+  const float2 e0 = unpack2(ext[0]), e1 = unpack2(ext[1]);
+  v[3] = e0.x + e0.y;
+  if (RB == 6) v[4] = e1.x + e1.y;
+  // lane l keeps sum l >> 2
+#pragma unroll
+  for (int h = 4, o = 16; h; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) {
+      const float got = __shfl_xor_sync(0xffffffffu, up ? v[k] : v[k + h], o);
+      v[k] = (up ? v[k + h] : v[k]) + got;
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 2);
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  float U[5];
+#pragma unroll
+  for (int b = 0; b < 5; ++b) {
+    const float p = __shfl_xor_sync(0xffffffffu, T, 1 << b);
+#pragma unroll
+    for (int i = 0; i < b; ++i) U[i] += __shfl_xor_sync(0xffffffffu, U[i], 1 << b);
+    U[b] = ((lane >> b) & 1) ? T : p;
+    T += p;
+  }
+  // one conversion and one store for the warp: lanes 4 k hold register bit k,
+  // lanes 4 b + 1 lane bit b (b = 5: the whole), lanes 4 b + 2 warp bit b
+  const int i = lane >> 2, kind = lane & 3;
+  float x = v[0];
+  int bit = i < RB ? ph.rb[i] : -1;
+  if (kind == 1) {
+    x = i == 0 ? U[0] : i == 1 ? U[1] : i == 2 ? U[2] : i == 3 ? U[3] : i == 4 ? U[4] : T;
+    bit = i < 5 ? ph.lanes[i] : i == 5 ? kMaxK : -1;
+  } else if (kind == 2) {
+    x = ((warp >> i) & 1) ? T : 0.f;
+    bit = i < lognt - 5 ? ph.warps[i] : -1;
+  }
+  if (kind < 3 && bit >= 0) row[bit] = (double)x;
 }
 
 // The pass's phases on one tile in shared memory, run by the 2^lognt threads
@@ -1508,13 +1570,18 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
         // one of which the readout spin is if it is a register bit at all (with
         // the spin's register bit found at run time and every pack tested for
         // it, this took 1300 cycles of a lone warp)
-        u64 acc[8];
+        u64 acc[8], ext[2] = {0ull, 0ull};
 #pragma unroll
         for (int i = 0; i < 8; ++i) acc[i] = 0ull;
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
           u64 &a = acc[(j & 3) | ((j >> (RB - 2)) << 2)];
-          a = add2(a, fma2(RE[j], RE[j], mul2(IM[j], IM[j])));
+          const u64 pr = fma2(RE[j], RE[j], mul2(IM[j], IM[j]));
+          a = add2(a, pr);
+          if constexpr (SITES) {  // and by the register bits between
+            if ((j >> 2) & 1) ext[0] = add2(ext[0], pr);
+            if (RB == 6 && ((j >> 3) & 1)) ext[1] = add2(ext[1], pr);
+          }
         }
         const int L = d.site_label;
         const uint32_t bit = d.site_thr >= 0 ? (uint32_t)(tid >> d.site_thr) & 1u
@@ -1526,35 +1593,7 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
           up += L == 0 ? v.y : hi ? v.x + v.y : 0.f;
           dn += L == 0 ? v.x : hi ? 0.f : v.x + v.y;
         }
-        if constexpr (SITES) {
-          // per tile bit, the weight with that bit up: register bits from the
-          // packs, thread-index bits the thread's whole sum
-          float tsum = 0.f, ureg[RB];
-#pragma unroll
-          for (int q = 0; q < RB; ++q) ureg[q] = 0.f;
-#pragma unroll
-          for (int j = 0; j < NP; ++j) {
-            const float2 pr = unpack2(fma2(RE[j], RE[j], mul2(IM[j], IM[j])));
-            const float sj = pr.x + pr.y;
-            tsum += sj;
-            ureg[0] += pr.y;
-#pragma unroll
-            for (int i = 0; i < RB - 1; ++i)
-              if ((j >> i) & 1) ureg[1 + i] += sj;
-          }
-          uint32_t tbits = 0;
-          for (int b = 0; b < 5; ++b) tbits |= ((uint32_t)(tid >> b) & 1u) << ph.lanes[b];
-          for (int b = 0; b < lognt - 5; ++b) tbits |= ((uint32_t)(tid >> (5 + b)) & 1u) << ph.warps[b];
-#pragma unroll
-          for (int q = 0; q < kMaxK; ++q) {
-            float v = ((tbits >> q) & 1u) ? tsum : 0.f;
-#pragma unroll
-            for (int k2 = 0; k2 < RB; ++k2)
-              if (ph.rb[k2] == q) v = ureg[k2];
-            warp_site_sum<float>(v, q, s_w);
-          }
-          warp_site_sum<float>(tsum, kMaxK, s_w);
-        }
+        if constexpr (SITES) site_sums<RB>(acc, ext, ph, tid, lognt, s_w);
         ++k;
       }
       ++st;
@@ -1695,7 +1734,7 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
                                              sw2::SyncBlock{}, RE, IM, psi);
   if constexpr (!DIRECT) sw2::store_tile<RB>(psi, base, d, tid, lognt, tile2);
   if constexpr (SITES)
-    if (d.has_reduce) write_site_partials(d, M, base, s_w, jp.psites);
+    if (d.has_reduce) write_site_partials(d, M, base, s_w, jp.psites, tid, nt, blockIdx.x, gridDim.x);
   if (d.has_reduce) reduce_finalize((double)up, (double)dn, jp, false);
 }
 

@@ -151,10 +151,8 @@ __device__ __forceinline__ void pipe_finalize(const double2 *partials, unsigned 
   }
 }
 
-// One sweep (complex64, plain storage, spin-1 readout) with 2^(K-RB) = 128
-// threads per compute group.  (A sweep that takes the all-site readout runs
-// sweep2_kernel's readout variant: under this kernel's 224-register budget
-// the readout's sums spill, measured 8 % slower per step at M = 30.)
+// One sweep (complex64, plain storage) with 2^(K-RB) = 128 threads per compute
+// group.
 //   BATCH = false: one job; jobs[0] holds its pointers (gate tables,
 //     partials, ticket, series), psi1, sops1, qdiag1 and dtab1 its amplitudes,
 //     resolved ops and diagonal-phase tables; the units are its tiles, and the last block to finish combines
@@ -174,11 +172,12 @@ __device__ __forceinline__ void pipe_finalize(const double2 *partials, unsigned 
 // many gates a phase (kPipeDense: walks over the register-bit pairs) and with
 // few (kPipeSparse: a jump to each gate's code; most pairs of a walk would be
 // skipped, and the whole walk's code competes for the instruction cache with
-// the producer's).  Measured with walks against jumps: 25-spin dipolar star
+// the producer's).  kPipeSites: a reducing pass that takes the all-site readout,
+// with or without the diagonal op.  Measured with walks against jumps: 25-spin dipolar star
 // (8.7 gates a phase) 18.3 against 21.8 ms for six steps, 26-spin ladder (5.4)
 // 24.5 against 22.5 ms for twenty; the line lies between.
 constexpr int kPipeDenseGates = 7;
-enum { kPipeSparse = 0, kPipeDense = 1, kPipeDiag = 2 };
+enum { kPipeSparse = 0, kPipeDense = 1, kPipeDiag = 2, kPipeSites = 3 };
 constexpr int kPipeBatchOps = kMaxPassOps / 3;  // resolved ops of a pass, per buffer (batches)
 static_assert(sizeof(JobPtrs) % 8 == 0, "job pointers copied as 8-byte words");
 
@@ -199,6 +198,7 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
   __shared__ __align__(16) JobPtrs s_job[BATCH ? 3 : 1];
   __shared__ __align__(8) uint64_t s_full[3], s_done[3];
   __shared__ double s_up[2][NW], s_dn[2][NW];
+  __shared__ double s_w[VAR == kPipeSites ? 2 * NW * kSiteSlots : 1];
   __shared__ int s_last;
 
   const int tid = threadIdx.x;
@@ -301,7 +301,8 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
     const uint64_t *const qdiag =
         reinterpret_cast<const uint64_t *>(reinterpret_cast<const char *>(qdiag1) + joff);
     const uint64_t *const dtab = reinterpret_cast<const uint64_t *>(reinterpret_cast<const char *>(dtab1) + joff);
-    if (VAR == kPipeDiag && !probe) sw2::diag_fields(d, base, gt, LOGNT, M, qdiag, sH[g]);
+    if ((VAR == kPipeDiag || (VAR == kPipeSites && d.diag >= 0)) && !probe)
+      sw2::diag_fields(d, base, gt, LOGNT, M, qdiag, sH[g]);
     const bool late = !pipe::mbar_wait(a_full + 8u * b, (i / 3u) & 1u, err);
     if (pipe::group_any(late, bar, NT)) {
       if (gt == 0) atomicExch(err, 1);
@@ -313,8 +314,9 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
     const ROpRes *ops = BATCH ? s_op + kPipeBatchOps * b : s_op;
     float up = 0.f, dn = 0.f;
     sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
-    sw2::run_phases<RB, false, false, sw2::kInPlace, VAR != kPipeSparse, VAR == kPipeDiag>(
-        tiles + b * TA, d, s_ph, ops, base, gt, LOGNT, dtab, up, dn, sH[g], nullptr, sync, RE, IM, nullptr);
+    double *const sw = VAR == kPipeSites ? s_w + g * NW * kSiteSlots : nullptr;
+    sw2::run_phases<RB, VAR == kPipeSites, false, sw2::kInPlace, VAR != kPipeSparse, VAR >= kPipeDiag>(
+        tiles + b * TA, d, s_ph, ops, base, gt, LOGNT, dtab, up, dn, sH[g], sw, sync, RE, IM, nullptr);
     // run_phases ends with the group's barrier: the tile is finished
     if (!d.has_reduce) {
       if (gt == 0) pipe::mbar_arrive(a_done + 8u * b);
@@ -324,6 +326,9 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
     // buffer goes back after the group's barrier below, once every thread
     // has read the job's reduction pointers from its slot
     double2 *const partials = js->partials;
+    // the weights by spin, published by run_phases' last barrier; the barrier
+    // below keeps them until every thread has read its columns
+    if constexpr (VAR == kPipeSites) write_site_partials(d, M, base, sw, js->psites, gt, NT, tile, T);
     double pu = (double)up, pv = (double)dn;
     for (int o = 16; o; o >>= 1) {
       pu += __shfl_xor_sync(0xffffffffu, pu, o);
