@@ -60,9 +60,41 @@ __device__ __forceinline__ void gate_combo(double (&re)[32], double (&im)[32], i
 
 // A phase op staged in shared memory with its FP64 gate coefficients.
 struct SOpD {
-  uint8_t kind, combo, arg, pad[5];
+  uint8_t kind, combo, arg, pad;
+  uint32_t tab;  // diagonal op: offset of its variant's table
   double t, s;
 };
+
+// The diagonal op on a complex128 tile, as sw2::diag_tile: Theta from the tables
+// and the outer fields (exact), two amplitudes a turn of the loop, out of line.
+// FP64 bound (sincospi). Against Theta walked over the phase's own register bits,
+// unrolled over 32 amplitudes with the K x K table staged by every block: ten
+// steps of the 20-spin star 13.83 -> 13.73 ms, the 14-spin ladder as it was.
+__device__ __noinline__ void diag_tile(double2 *tile16, const uint64_t *__restrict__ tab, const uint64_t *sH, int K,
+                                       int tid, int lognt) {
+  constexpr int RB = 5;
+  const uint64_t *__restrict__ tthr = tab + (1 << RB) + tid;
+  uint64_t g[RB], base = sH[K] + tthr[0];
+#pragma unroll
+  for (int k = 0; k < RB; ++k) g[k] = sH[lognt + k] + tthr[(size_t)(k + 1) << lognt];
+  for (int b = 0; b < lognt; ++b) base += ((tid >> b) & 1) ? sH[b] : (0ull - sH[b]);
+  uint32_t ds[RB];
+#pragma unroll
+  for (int k = 0; k < RB; ++k) base -= g[k], g[k] += g[k], ds[k] = slot(1u << (lognt + k));
+  const uint32_t o0 = slot((uint32_t)tid);
+#pragma unroll 1
+  for (int e = 0; e < (1 << RB); e += 2) {
+    uint64_t lin = base;
+    uint32_t o = o0;
+#pragma unroll
+    for (int k = 1; k < RB; ++k)
+      if ((e >> k) & 1) lin += g[k], o ^= ds[k];
+    const double2 a = tile16[o], b = tile16[o ^ ds[0]];
+    const double2 p = cis_turns(lin + tab[e], 0.0), q = cis_turns(lin + g[0] + tab[e + 1], 0.0);
+    tile16[o] = cmul(a, p);
+    tile16[o ^ ds[0]] = cmul(b, q);
+  }
+}
 
 }  // namespace sw2d
 
@@ -73,11 +105,8 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
   constexpr int RB = 5, NA = 32;
   const JobPtrs jp = jobs[blockIdx.y];
   double2 *__restrict__ psi = static_cast<double2 *>(jp.psi);
-  const uint64_t *__restrict__ qdiag = jp.qdiag;
   extern __shared__ __align__(16) double2 tile16[];
-  __shared__ uint64_t sH[kMaxK];
-  __shared__ uint64_t sQ[kMaxK * kMaxK];
-  __shared__ uint64_t sOut;
+  __shared__ uint64_t sH[kMaxK + 1];
   __shared__ PhaseDesc s_ph[kMaxPassPhases];
   __shared__ sw2d::SOpD s_op[kMaxPassOps];
   const int K = d.K, tid = threadIdx.x, nt = blockDim.x;
@@ -90,7 +119,8 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
   for (int i = tid; i < d.nrops; i += nt) {
     const ROp r = rops[d.rop0 + i];
     sw2d::SOpD o;
-    o.kind = r.kind, o.combo = r.combo, o.arg = r.arg;
+    o.kind = r.kind, o.combo = r.combo, o.arg = r.arg, o.pad = 0;
+    o.tab = r.kind == OP_DIAG ? (uint32_t)r.coef : 0u;
     o.t = 0.0, o.s = 0.0;
     if (r.kind == OP_GATE) {
       const GateCoef g = jp.coefs[r.coef];
@@ -98,6 +128,7 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
     }
     s_op[i] = o;
   }
+  if (d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   grid_wait();
   // ---- global -> shared: 16-byte async copies, amplitude a = tid + nt * e,
   // e in Gray-code order in runs of eight (as in the complex64 kernel)
@@ -150,7 +181,6 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
   __syncthreads();
 
   double up = 0.0, dn = 0.0;
-  const int nout = M - K;
   const char *tb = reinterpret_cast<const char *>(tile16);
   char *tw = reinterpret_cast<char *>(tile16);
   for (int p = 0; p < d.nphases; ++p) {
@@ -166,84 +196,7 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
     for (int k = 0; k < 5; ++k) t0 |= ((uint32_t)(tid >> k) & 1u) << ph.lanes[k];
     for (int k = 0; k < lognt - 5; ++k) t0 |= ((uint32_t)(tid >> (5 + k)) & 1u) << ph.warps[k];
     if (ph.nops == 1 && s_op[o0].kind == OP_DIAG) {
-      // e^{-i tau D} amplitude by amplitude in shared memory, Theta walked in
-      // Gray-code order over the register bits (as in the complex64 kernel)
-      const uint64_t *q = qdiag + (size_t)s_op[o0].arg * M * M;
-      if (tid < K) {
-        const int pp = d.tile_pos[tid];
-        uint64_t h = 0;
-        for (int o = 0; o < nout; ++o) {
-          const int po = d.outer_pos[o];
-          const uint64_t v = q[pp * M + po];
-          h += ((base >> po) & 1ull) ? v : (0ull - v);
-        }
-        sH[tid] = h;
-      } else if (tid == K) {
-        uint64_t sacc = 0;
-        for (int o = 0; o < nout; ++o)
-          for (int o2 = o + 1; o2 < nout; ++o2) {
-            const int pa = d.outer_pos[o], pb = d.outer_pos[o2];
-            const uint64_t v = q[pa * M + pb];
-            sacc += (((base >> pa) ^ (base >> pb)) & 1ull) ? (0ull - v) : v;
-          }
-        sOut = sacc;
-      }
-      for (int w = tid; w < K * K; w += nt) sQ[w] = q[d.tile_pos[w / K] * M + d.tile_pos[w % K]];
-      __syncthreads();
-      uint32_t isreg = 0;
-      for (int k = 0; k < RB; ++k) isreg |= 1u << ph.rb[k];
-      uint64_t th0 = sOut;
-      for (int x = 0; x < K; ++x) {
-        if ((isreg >> x) & 1u) continue;
-        const uint32_t bx = (t0 >> x) & 1u;
-        th0 += bx ? sH[x] : (0ull - sH[x]);
-        for (int y = x + 1; y < K; ++y) {
-          if ((isreg >> y) & 1u) continue;
-          th0 += (bx ^ ((t0 >> y) & 1u)) ? (0ull - sQ[x * K + y]) : sQ[x * K + y];
-        }
-      }
-      uint64_t G[RB], Qr[RB][RB], F[RB];
-#pragma unroll
-      for (int k = 0; k < RB; ++k) {
-        const int rk = ph.rb[k];
-        uint64_t gk = sH[rk];
-        for (int x = 0; x < K; ++x) {
-          if ((isreg >> x) & 1u) continue;
-          gk += ((t0 >> x) & 1u) ? sQ[x * K + rk] : (0ull - sQ[x * K + rk]);
-        }
-        G[k] = gk;
-      }
-#pragma unroll
-      for (int k = 0; k < RB; ++k)
-#pragma unroll
-        for (int l = 0; l < RB; ++l)
-          Qr[k][l] = k == l ? 0ull : sQ[ph.rb[k < l ? k : l] * K + ph.rb[k < l ? l : k]];
-      uint64_t th = th0;
-#pragma unroll
-      for (int k = 0; k < RB; ++k) {
-        th -= G[k];
-        F[k] = G[k];
-#pragma unroll
-        for (int l = 0; l < RB; ++l) {
-          if (l == k) continue;
-          F[k] -= Qr[k][l];
-          if (l > k) th += Qr[k][l];
-        }
-      }
-      uint32_t sl = s0;
-#pragma unroll
-      for (int g = 0; g < NA; ++g) {
-        if (g) {
-          const int k = sw2::ctz5(g);
-          const bool was_up = ((((g - 1) ^ ((g - 1) >> 1)) >> k) & 1) != 0;
-          th += was_up ? (0ull - 2ull * F[k]) : 2ull * F[k];
-#pragma unroll
-          for (int l = 0; l < RB; ++l)
-            if (l != k) F[l] += was_up ? (0ull - 2ull * Qr[l][k]) : 2ull * Qr[l][k];
-          sl ^= sm[k];
-        }
-        tile16[sl] = cmul(tile16[sl], cis_turns(th, 0.0));
-      }
+      sw2d::diag_tile(tile16, jp.dtab + s_op[o0].tab, sH, K, tid, lognt);
       __syncthreads();
       continue;
     }
