@@ -1,9 +1,8 @@
 // sweep2d.cuh -- register-blocked tile sweep for complex128 states (sm_103a).
 //
 // The complex128 counterpart of sweep2_kernel: the same pass programs (phases
-// of register bits, gates as three shears per plane, the diagonal phase by
-// Gray-code field updates, the fused P/norm readout), with 32 FP64 amplitudes
-// per thread and 16-byte shared-memory slots.  Bound by the FP64 pipe.
+// of register bits, gates as three shears per plane, the tabulated diagonal op,
+// the fused P/norm readout), with 32 FP64 amplitudes per thread and 16-byte shared-memory slots.  Bound by the FP64 pipe.
 #pragma once
 #include "kernels.cuh"
 
