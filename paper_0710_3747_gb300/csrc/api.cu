@@ -295,13 +295,14 @@ extern "C" int spinrp_system_set_regbits(spinrp_system *sys, int rb) {
 // (at most M) of least modelled cost, sweeps per step x max(2^K, njobs 2^M /
 // kModelSMs): a sweep lasts about one tile's work while the tiles do not fill
 // the SMs, and about the state's share per SM once they do.  Ties go to 13,
-// then 12, then 14.  Measured on GB300 against the other widths: ladders of
-// 14, 18, 22, 24 and 30 spins, dipolar stars of 16, 20 and 22 spins, and the
-// batch of 12..22-spin stars (the model's pick was the fastest, or within
-// 2 %, in every case).  Where 13-spin tiles run as the pipelined sweep
+// then 12, then 14.  Measured on GB300, us per step at K 12 / 13 / 14: ladders
+// of 14 spins 14.9 / 19.0 / 16.0, 18 18.5 / 22.9 / 34.4, 22 87.9 / 63.6 / 80.2,
+// 24 306.5 / 296.7 / 278.0, 26 1172 / 1069 / 1397; dipolar stars of 16 45.6 /
+// 58.7 / 90.4, 20 106.6 / 139.2 / 125.9, 22 358.5 / 318.3 / 363.4, 24 1421 /
+// 1339 / 1436 (the model's pick is the fastest but on the 24-spin ladder, 6 %).  Where 13-spin tiles run as the pipelined sweep
 // (pipe_kernel: six register bits, plain storage, at least four units per
-// SM) a sweep costs kPipeSweepCost of the model's sweep: measured per-sweep
-// time of the pipelined 13-spin sweep over the 14-spin one 0.58, 0.59 and
+// SM) a sweep costs kPipeSweepCost of the model's sweep: per-sweep time measured
+// (before the register programs' walks) of the pipelined 13-spin sweep over the 14-spin one 0.58, 0.59 and
 // 0.72 on dipolar stars of 23, 24 and 26 spins, 0.48, 0.70 and 0.67 on
 // ladders of 24, 26 and 28 spins, 0.49 and 0.47 on batches of 383 and 363
 // dipolar stars of 20 and 21 spins (8 sweeps per step against 4: 29.2
