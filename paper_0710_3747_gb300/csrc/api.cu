@@ -398,7 +398,7 @@ struct PassSet {
   // per phase (a walk over the register-bit pairs pays from kPipeDenseGates on)
   int variant(int pass, bool sites) const {
     const PassDesc &d = desc[pass];
-    return sites ? kPipeSites : d.diag >= 0 ? kPipeDiag : d.nops >= kPipeDenseGates * d.nphases ? kPipeDense : kPipeSparse;
+    return sites ? kPipeSites : d.diag ? kPipeDiag : d.nops >= kPipeDenseGates * d.nphases ? kPipeDense : kPipeSparse;
   }
 };
 
@@ -511,7 +511,6 @@ static void build_passes(const Plan &p, bool has_diag, PassSet *ps) {
     std::vector<int> in_spin(M, -1), out_spin(M, -1);  // physical position -> spin
     for (int q = 0; q < M; ++q) in_spin[Lin[q]] = q, out_spin[Lout[q]] = q;
     d.relabel = 0;
-    d.diag = -1;
     for (int qo = 0; qo < K; ++qo) {
       d.tile_pos[qo] = (uint8_t)tpos[qo];
       const int spin = out_spin[tpos[qo]];
@@ -557,7 +556,7 @@ static void build_passes(const Plan &p, bool has_diag, PassSet *ps) {
     op.kind = OP_DIAG;
     op.arg = (uint8_t)variant;
     push(pass, op);
-    ps->desc[pass].diag = variant;
+    ps->desc[pass].diag |= 1 << variant;
   };
   auto reduce = [&](int pass) {
     Op op{};
@@ -978,7 +977,7 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
       }
     }
     // the diagonal op's tables (the same tile bits in every pass that has one)
-    if (d.diag >= 0) {
+    if (d.diag) {
       DiagTab t;
       t.rb = (uint8_t)RB, t.L = (uint8_t)(K - RB);
       t.words = (1 << RB) + (1 + RB) * (1 << (K - RB));
@@ -2592,7 +2591,9 @@ extern "C" int spinrp_system_plan_check(const spinrp_system *sys, int prec, doub
           ++g;
         } else if (r.kind == OP_DIAG) {
           if (ph.nops != 1) return fail(SPINRP_EINVAL, "plan_check: diagonal op shares a phase");
-          if (d.diag < 0 || r.coef != r.arg * ps.tab.words || ps.tab.rb != ps.rb || ps.tab.L != K - ps.rb)
+          if (!((d.diag >> r.arg) & 1))
+            return fail(SPINRP_EINVAL, "plan_check: pass %zu: no outer fields for a diagonal op's variant", pi);
+          if (r.coef != r.arg * ps.tab.words || ps.tab.rb != ps.rb || ps.tab.L != K - ps.rb)
             return fail(SPINRP_EINVAL, "plan_check: pass %zu: diagonal table", pi);
           check_diag(B, r.arg);
         } else {

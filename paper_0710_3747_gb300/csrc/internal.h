@@ -56,7 +56,8 @@ struct PassDesc {
   int32_t rop0;         //   first op
   int32_t nrops;        //   and number of ops
   uint8_t store_bit[kMaxK];  // store: output tile bit (1..K-1) of each chunk-index bit
-  int32_t diag;         // S^zS^z variant of the pass's diagonal ops (0: dt/2, 1: dt), -1 without any
+  int32_t diag;         // S^zS^z variants of the pass's diagonal ops: bit 0 dt/2, bit 1 dt (the first sweep of
+                        // a one-segment plan has both), 0 without any
   // a direct pass's first phase loads its subcubes from the state and its last
   // phase stores them there (tile bits 0 and 1, in the output order for the
   // store, are register bits 1 and 2); physical positions of the thread-index
@@ -132,6 +133,10 @@ struct ROp {
   uint8_t pad;
   int32_t coef;
 };
+
+// A pass's outer spins act on its tile as fields, one per tile bit, and a part of
+// their own, for each variant of the diagonal op: entries of one variant.
+constexpr int kFieldStride = kMaxK + 1;
 
 struct GateCoef;
 

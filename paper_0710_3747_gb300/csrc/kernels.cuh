@@ -1026,39 +1026,44 @@ __device__ __forceinline__ uint32_t thread_origin(const PhaseDesc &ph, int tid, 
   return t0;
 }
 
-// Fields of the outer spins on a tile's bits, sH[t] = sum_o sigma_o q_to, and
-// their own part of Theta, sH[K] (exact modulo 2^64), by the 2^lognt threads
-// tid of the group: eight lanes share each entry, so the loads of a row are in
-// flight together.  The group's next barrier publishes them.
+// For each variant v of the pass's diagonal ops: fields of the outer spins on a
+// tile's bits, sH[v kFieldStride + t] = sum_o sigma_o q_to, and their own part of
+// Theta at t = K (exact modulo 2^64), by the 2^lognt threads tid of the group:
+// eight lanes share each entry, so the loads of a row are in flight together.
+// The group's next barrier publishes them.
 __device__ __forceinline__ void diag_fields(const PassDesc &d, uint64_t base, int tid, int lognt, int M,
                                             const uint64_t *__restrict__ qdiag, uint64_t *sH) {
   const int K = d.K, nout = M - K, part = tid & 7;
-  const uint64_t *__restrict__ q = qdiag + (size_t)d.diag * M * M;
-  for (int t0 = 0; t0 <= K; t0 += 1 << (lognt - 3)) {
-    const int t = t0 + (tid >> 3);
-    uint64_t v = 0;
-    if (t < K) {
-      const int row = d.tile_pos[t] * M;
-      for (int o = part; o < nout; o += 8) {
-        const int po = d.outer_pos[o];
-        const uint64_t x = q[row + po];
-        v += ((base >> po) & 1ull) ? x : (0ull - x);
-      }
-    } else if (t == K) {
-      for (int o = part; o < nout; o += 8) {
-        const int pa = d.outer_pos[o];
-        uint64_t r = 0;
-        for (int o2 = o + 1; o2 < nout; ++o2) {
-          const int pb = d.outer_pos[o2];
-          const uint64_t x = q[pa * M + pb];
-          r += ((base >> pb) & 1ull) ? x : (0ull - x);
+#pragma unroll 1
+  for (int var = 0; var < 2; ++var) {
+    if (!((d.diag >> var) & 1)) continue;
+    const uint64_t *__restrict__ q = qdiag + (size_t)var * M * M;
+    for (int t0 = 0; t0 <= K; t0 += 1 << (lognt - 3)) {
+      const int t = t0 + (tid >> 3);
+      uint64_t v = 0;
+      if (t < K) {
+        const int row = d.tile_pos[t] * M;
+        for (int o = part; o < nout; o += 8) {
+          const int po = d.outer_pos[o];
+          const uint64_t x = q[row + po];
+          v += ((base >> po) & 1ull) ? x : (0ull - x);
         }
-        v += ((base >> pa) & 1ull) ? r : (0ull - r);
+      } else if (t == K) {
+        for (int o = part; o < nout; o += 8) {
+          const int pa = d.outer_pos[o];
+          uint64_t r = 0;
+          for (int o2 = o + 1; o2 < nout; ++o2) {
+            const int pb = d.outer_pos[o2];
+            const uint64_t x = q[pa * M + pb];
+            r += ((base >> pb) & 1ull) ? x : (0ull - x);
+          }
+          v += ((base >> pa) & 1ull) ? r : (0ull - r);
+        }
       }
-    }
 #pragma unroll
-    for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (part == 0 && t <= K) sH[t] = v;
+      for (int o = 4; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (part == 0 && t <= K) sH[var * kFieldStride + t] = v;
+    }
   }
 }
 
@@ -1514,7 +1519,7 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
     // the phase's first step, and the coefficients of its first gate if it is a round
     uint32_t step = ORIENT ? 0u : d.steps[st];
     if (DIAG && (ORIENT ? ph.nops == 1 && s_op[o0].kind == OP_DIAG : (step & kStepDiag) != 0)) {
-      diag_tile<RB, ORIENT>(tile2, dtab + s_op[o0].tab, sH, d.K, tid, lognt, d.black_tile, outer_par);
+      diag_tile<RB, ORIENT>(tile2, dtab + s_op[o0].tab, sH + s_op[o0].arg * kFieldStride, d.K, tid, lognt, d.black_tile, outer_par);
       sync();
       ++st;
       continue;
@@ -1696,7 +1701,7 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   const JobPtrs jp = jobs[blockIdx.y];
   float2 *__restrict__ psi = one ? psi1 : static_cast<float2 *>(jp.psi);
   extern __shared__ __align__(16) float2 tile2[];
-  __shared__ uint64_t sH[kMaxK + 1];
+  __shared__ uint64_t sH[2 * kFieldStride];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
   __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 2];  // coefficients are read ahead
   __shared__ double s_w[SITES ? kMaxWarps * kSiteSlots : 1];
@@ -1718,14 +1723,14 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
     const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
     for (int i = tid; i < d.nrops; i += nt) sw2::cp_async16(a_op + 16u * i, so + i);
   }
-  if (chained && d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
+  if (chained && d.diag) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   grid_wait();
   sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
   if constexpr (DIRECT) sw2::load_direct<RB>(psi, base, d, tid, lognt, RE, IM);
   else sw2::load_tile<RB>(psi, base, d, tid, lognt, (uint32_t)__cvta_generic_to_shared(tile2));
   if (ahead && blockIdx.x + ahead < gridDim.x)
     sw2::prefetch_tile<RB>(psi, sw2::tile_origin(blockIdx.x + ahead, d, M), d, tid, lognt);
-  if (!chained && d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
+  if (!chained && d.diag) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   sw2::cp_async_wait_all();
   __syncthreads();
 
@@ -1763,7 +1768,7 @@ resident_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ Reside
   extern __shared__ __align__(16) float2 tile2[];
   PhaseDesc *s_ph = reinterpret_cast<PhaseDesc *>(tile2 + (size_t(1) << M));
   ROpRes *s_op = reinterpret_cast<ROpRes *>(s_ph + nph);
-  __shared__ uint64_t sH[kMaxK + 1];
+  __shared__ uint64_t sH[2 * kFieldStride];
   __shared__ double s_up[8], s_dn[8];
   const int tid = threadIdx.x, nt = blockDim.x;
   const int lognt = M - RB;
@@ -1777,7 +1782,7 @@ resident_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ Reside
     const uint32_t a_op = (uint32_t)__cvta_generic_to_shared(s_op);
     for (int i = tid; i < nrops; i += nt) sw2::cp_async16(a_op + 16u * i, jp.sops + i);
   }
-  for (int i = tid; i <= M; i += nt) sH[i] = 0;  // no outer spins: no fields
+  for (int i = tid; i < 2 * kFieldStride; i += nt) sH[i] = 0;  // no outer spins: no fields
   sw2::cp_async_wait_all();
   __syncthreads();
   const int64_t slot0 = *jp.step;

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(256)
 persist_kernel(const PersistPlan *__restrict__ plan, unsigned long long *queue, unsigned *done, int *err,
                unsigned ahead) {
   extern __shared__ __align__(16) float2 tile2[];
-  __shared__ uint64_t sH[kMaxK + 1];
+  __shared__ uint64_t sH[2 * kFieldStride];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
   __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 2];  // coefficients are read ahead
   __shared__ __align__(16) PassDesc s_d;
@@ -273,7 +273,7 @@ persist_kernel(const PersistPlan *__restrict__ plan, unsigned long long *queue, 
     if (ahead && r + ahead < G.tiles) sw2::prefetch_tile<RB>(psi, sw2::tile_origin(r + ahead, d, M), d, tid, lognt);
     pq::load_tile_cg<RB>(psi, base, d, tid, lognt, tile2);
     if (tid == 0) next = atomicAdd(queue, 1ull);
-    if (d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
+    if (d.diag) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
     sw2::cp_async_wait_all();
     __syncthreads();
     float up = 0.f, dn = 0.f;

@@ -191,7 +191,7 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
   constexpr uint32_t TA = 1u << K; // amplitudes per tile buffer
   static_assert(NT == 128, "groups are warpgroups");
   extern __shared__ __align__(16) float2 tiles[];
-  __shared__ uint64_t sH[2][kMaxK + 1];
+  __shared__ uint64_t sH[2][2 * kFieldStride];
   __shared__ __align__(16) PhaseDesc s_ph[kMaxPassPhases];
   // one job: the pass's ops; BATCH: three slices of kPipeBatchOps, one per buffer
   __shared__ __align__(16) ROpRes s_op[kMaxPassOps + 2];  // coefficients are read ahead
@@ -301,7 +301,7 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
     const uint64_t *const qdiag =
         reinterpret_cast<const uint64_t *>(reinterpret_cast<const char *>(qdiag1) + joff);
     const uint64_t *const dtab = reinterpret_cast<const uint64_t *>(reinterpret_cast<const char *>(dtab1) + joff);
-    if ((VAR == kPipeDiag || (VAR == kPipeSites && d.diag >= 0)) && !probe)
+    if ((VAR == kPipeDiag || (VAR == kPipeSites && d.diag)) && !probe)
       sw2::diag_fields(d, base, gt, LOGNT, M, qdiag, sH[g]);
     const bool late = !pipe::mbar_wait(a_full + 8u * b, (i / 3u) & 1u, err);
     if (pipe::group_any(late, bar, NT)) {

@@ -105,7 +105,7 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
   const JobPtrs jp = jobs[blockIdx.y];
   double2 *__restrict__ psi = static_cast<double2 *>(jp.psi);
   extern __shared__ __align__(16) double2 tile16[];
-  __shared__ uint64_t sH[kMaxK + 1];
+  __shared__ uint64_t sH[2 * kFieldStride];
   __shared__ PhaseDesc s_ph[kMaxPassPhases];
   __shared__ sw2d::SOpD s_op[kMaxPassOps];
   const int K = d.K, tid = threadIdx.x, nt = blockDim.x;
@@ -127,7 +127,7 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
     }
     s_op[i] = o;
   }
-  if (d.diag >= 0) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
+  if (d.diag) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   grid_wait();
   // ---- global -> shared: 16-byte async copies, amplitude a = tid + nt * e,
   // e in Gray-code order in runs of eight (as in the complex64 kernel)
@@ -195,7 +195,7 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
     for (int k = 0; k < 5; ++k) t0 |= ((uint32_t)(tid >> k) & 1u) << ph.lanes[k];
     for (int k = 0; k < lognt - 5; ++k) t0 |= ((uint32_t)(tid >> (5 + k)) & 1u) << ph.warps[k];
     if (ph.nops == 1 && s_op[o0].kind == OP_DIAG) {
-      sw2d::diag_tile(tile16, jp.dtab + s_op[o0].tab, sH, K, tid, lognt);
+      sw2d::diag_tile(tile16, jp.dtab + s_op[o0].tab, sH + s_op[o0].arg * kFieldStride, K, tid, lognt);
       __syncthreads();
       continue;
     }
