@@ -447,6 +447,7 @@ struct spinrp_state {
   int64_t *stage_idx = nullptr;
   JobPtrs *d_job = nullptr;   // this state's pointer table (one job)
   JobPtrs hjob{};             // the same, host copy (passed with each sweep launch)
+  unsigned per_sm[2] = {0, 0};  // one-tile-per-block sweep blocks an SM holds (1: with the all-site readout)
   unsigned prefetch_ahead = 0;  // L2 prefetch distance of the register-blocked sweep
   unsigned pipe_blocks = 0;   // blocks of the pipelined sweep, 0 when the plan does not take it
   bool pipe_req = true;       // pipelined sweeps where the plan takes them
@@ -1114,6 +1115,9 @@ static void free_state(spinrp_state *st) {
 constexpr size_t kResidentMaxSmem = size_t(223) * 1024;
 constexpr size_t kPipeSmem = size_t(3) << 16;  // pipe_kernel<6, 13, *>: three 64 KiB tile buffers
 
+// Threads of a plain-sweep block: one a plane of a gate's pairs.
+static int plain_threads(int K) { return std::min(512, std::max(32, 1 << K >> 1)); }
+
 template <typename R>
 static int set_smem_limits() {
   // the widest tile of this precision (2^14 c64 or 2^13 c128 = 128 KiB)
@@ -1154,32 +1158,50 @@ static int set_smem_limits() {
   return SPINRP_OK;
 }
 
-// Register-blocked sweep blocks resident on the whole device at once (the L2
-// prefetch distance); 0 when the query fails.
-static unsigned sweep2_resident(int prec, int rb, int K, bool oriented) {
-  int dev = 0, sms = 0, per = 0;
+static int device_sms() {
+  int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  const size_t smem = (prec == SPINRP_C64 ? size_t(8) : size_t(16)) << K;
-  const cudaError_t e =
-      prec != SPINRP_C64
-          ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2d_kernel, 1 << (K - 5), smem)
-      : rb == 6 ? (oriented ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<6, false, true, false>,
-                                                                            1 << (K - 6), smem)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<6, false, false, true>,
-                                                                            1 << (K - 6), smem))
-                : (oriented ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<5, false, true, false>,
-                                                                            1 << (K - 5), smem)
-                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, sweep2_kernel<5, false, false, true>,
-                                                                            1 << (K - 5), smem));
+  return sms;
+}
+
+// Blocks of a plan's one-tile-per-block sweep that an SM holds at once (sites:
+// of the sweep that takes the all-site readout); 0 when the query fails.
+static unsigned sweep_per_sm(int prec, const PassSet &ps, int K, bool sites) {
+  const bool c64 = prec == SPINRP_C64;
+  const size_t smem = (c64 ? size_t(8) : size_t(16)) << K;
+  int per = 0;
+  auto query = [&](auto *kernel, int threads) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, threads, smem);
+  };
+  cudaError_t e;
+  if (!ps.phased || (!c64 && sites)) {
+    const int nt = plain_threads(K);
+    e = c64 ? (sites ? query(sweep_kernel<float, true>, nt) : query(sweep_kernel<float, false>, nt))
+            : (sites ? query(sweep_kernel<double, true>, nt) : query(sweep_kernel<double, false>, nt));
+  } else if (!c64) {
+    e = query(sweep2d_kernel, 1 << (K - 5));
+  } else {
+    const int nt = 1 << (K - ps.rb);
+    switch ((ps.rb == 6 ? 4 : 0) | (sites ? 2 : 0) | (ps.oriented ? 1 : 0)) {
+      case 0: e = query(sweep2_kernel<5, false, false, true>, nt); break;
+      case 1: e = query(sweep2_kernel<5, false, true, false>, nt); break;
+      case 2: e = query(sweep2_kernel<5, true, false, true>, nt); break;
+      case 3: e = query(sweep2_kernel<5, true, true, false>, nt); break;
+      case 4: e = query(sweep2_kernel<6, false, false, true>, nt); break;
+      case 5: e = query(sweep2_kernel<6, false, true, false>, nt); break;
+      case 6: e = query(sweep2_kernel<6, true, false, true>, nt); break;
+      default: e = query(sweep2_kernel<6, true, true, false>, nt); break;
+    }
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
-  return (unsigned)(per * sms);
+  return (unsigned)per;
 }
 
 // Blocks of the pipelined sweep (pipe_kernel, one per SM) for the plan of
@@ -1323,7 +1345,10 @@ extern "C" int spinrp_state_create(const spinrp_system *sys, int prec, void *str
     free_state(st);
     return rc;
   }
-  if (st->ps.phased) st->prefetch_ahead = sweep2_resident(prec, st->ps.rb, st->plan.K, st->ps.oriented);
+  if (st->ps.phased) {
+    st->per_sm[0] = sweep_per_sm(prec, st->ps, st->plan.K, false);
+    st->prefetch_ahead = st->per_sm[0] * device_sms();
+  }
   st->pipe_blocks = pipe_grid(prec, st->plan, st->ps, st->M);
   if (st->ps.oriented) {
     st->orient_black = st->ps.black;
@@ -1543,6 +1568,7 @@ struct LaunchCtx {
   int rb = 5;                    // register bits of the register-blocked kernel
   bool oriented = false;         // oriented program and state (complex64)
   int sites = 0;                 // all-site readout after every reducing sweep
+  unsigned per_sm[2] = {0, 0};   // one-tile-per-block sweep blocks an SM holds (1: with the all-site readout)
   unsigned prefetch_ahead = 0;   // sweep blocks resident at once (L2 prefetch distance), 0 = off
   bool resident = false;         // whole state kept in shared memory for every step (resident_kernel)
   unsigned pipe_blocks = 0;      // > 0: one-job sweeps of the plan run as pipe_kernel on this many blocks
@@ -1596,11 +1622,12 @@ static int launch_resident(const LaunchCtx &c, cudaStream_t stream, int64_t step
 }
 
 // A sweep launch.  chained: it may start while the kernel before it on the
-// stream, a sweep too, still runs; the kernel stages its program and waits for
-// that one before it touches the state (grid_wait).  Not for the first sweep of
-// an evolve call: the tables it stages may have just been launched.  Takes part
-// of a sweep's launch and prologue off the chain (per step: 14-spin ladder 17.9
-// -> 16.9 us, complex128 37.7 -> 35.6; 17-spin star 62.3 -> 59.5).
+// stream still runs, once all of that one's blocks have seen the kernel before
+// them finish; the kernel stages its program and waits for the one before
+// (grid_wait) before it touches the state.  Not for the first sweep of an evolve
+// call: the tables it stages may have just been launched.  Takes a sweep's launch
+// and prologue off the chain (per step: 14-spin ladder 16.6 -> 15.1 us, complex128
+// 33.1 -> 26.1; 17-spin star 54.9 -> 49.9).
 template <typename... P, typename... A>
 static cudaError_t launch_sweep(bool chained, dim3 grid, unsigned threads, size_t smem, cudaStream_t stream,
                                 void (*kernel)(P...), A... args) {
@@ -1613,12 +1640,30 @@ static cudaError_t launch_sweep(bool chained, dim3 grid, unsigned threads, size_
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Whether a one-tile-per-block sweep of `blocks` blocks, `per` of which fit an
+// SM, is launched chained.  Its early blocks take what the running sweep leaves
+// free.  That is harmless where both sweeps fit side by side (blocks go to the
+// emptiest SMs) or where an SM holds no more blocks than an even spread gives it;
+// between, some SMs fill up with the next sweep while others get none of it, and
+// stay so from sweep to sweep.  Chained against not, us per step, 256-block
+// complex128 chains: 18 spins in 2^10 tiles (five an SM, both fit) 83.4 against
+// 88.7; 19 in 2^11 (three an SM) 119.7 against 85.5, so not chained; 20 in 2^12
+// (two an SM, an even spread) 147.8 against 149.4.  128 blocks, both sweeps fit:
+// complex128 stars of 15, 17, 19 spins 110 against 133, 539 against 556, 689
+// against 700; complex64 19-spin chain 15.9 against 17.8, four 17-spin stars 51.7
+// against 55.9.  complex64 sweeps of more blocks than SMs start after the sweep
+// before.
+static bool chain_pays(uint64_t blocks, unsigned per, bool c128) {
+  if (per == 0 || (!c128 && blocks > (uint64_t)kModelSMs)) return false;
+  return 2 * blocks <= (uint64_t)per * kModelSMs || (blocks + kModelSMs - 1) / kModelSMs >= per;
+}
+
 // Launch one sweep on `stream`; `live` launches are counted and profiled,
 // launches recorded into a graph are not.
 template <typename R>
 static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool live, bool chained) {
   const int K = c.K;
-  const int nt = std::min(512, std::max(32, 1 << K >> 1));  // plain sweep: a thread a plane
+  const int nt = plain_threads(K);
   const size_t smem = sizeof(typename CT<R>::T) << K;
   const dim3 grid(1u << (c.M - K), (unsigned)c.njobs);
   if (live) {
@@ -1628,11 +1673,7 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
   // the all-site sums are taken only in the sweep that reads P out; the
   // other sweeps of an all-site run are the plain ones
   const bool sites = c.sites && c.ps->desc[pass].has_reduce;
-  // one-tile-per-block sweeps of more blocks than SMs start after the sweep
-  // before: blocks let in early land where that one's blocks are not, and stay
-  // unevenly spread (20-spin star, 256 blocks: 160 us a step against 113).
-  // (At most two complex128 tiles share an SM: 138 us a sweep against 140.)
-  const bool few = (uint64_t)grid.x * grid.y <= (uint64_t)kModelSMs || sizeof(R) == 8;
+  const bool early = chained && chain_pays(grid.x * (uint64_t)grid.y, c.per_sm[sites], sizeof(R) == 8);
   if (sizeof(R) == 4 && c.v2)
   {
     const size_t sm2 = size_t(8) << K;
@@ -1666,8 +1707,8 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
       }
     } else {
 #define SW2(RB_, S_, O_, D_)                                                                          \
-  CUDA_TRY(launch_sweep(chained && few, grid, 1u << (K - RB_), sm2, stream, sweep2_kernel<RB_, S_, O_, D_>, c.jobs, \
-                        psi1, sops1, pd, c.phases, c.M, ahead, chained && few))
+  CUDA_TRY(launch_sweep(early, grid, 1u << (K - RB_), sm2, stream, sweep2_kernel<RB_, S_, O_, D_>, c.jobs, \
+                        psi1, sops1, pd, c.phases, c.M, ahead, early))
       switch (code | (pd.direct ? 8 : 0)) {
         case 0: SW2(5, false, false, false); break;
         case 1: SW2(5, false, true, false); break;
@@ -1687,12 +1728,12 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
   }
   else if (sizeof(R) == 8 && c.v2 && !sites)
     // complex128 register-blocked (the all-site sums run in the plain kernel)
-    CUDA_TRY(launch_sweep(chained && few, grid, 1u << (K - 5), smem, stream, sweep2d_kernel, c.jobs, c.ps->desc[pass], c.phases,
+    CUDA_TRY(launch_sweep(early, grid, 1u << (K - 5), smem, stream, sweep2d_kernel, c.jobs, c.ps->desc[pass], c.phases,
                           c.rops, c.M, c.prefetch_ahead));
   else if (sites)
-    CUDA_TRY(launch_sweep(chained && few, grid, nt, smem, stream, sweep_kernel<R, true>, c.jobs, c.passes + pass, c.ops, c.M));
+    CUDA_TRY(launch_sweep(early, grid, nt, smem, stream, sweep_kernel<R, true>, c.jobs, c.passes + pass, c.ops, c.M));
   else
-    CUDA_TRY(launch_sweep(chained && few, grid, nt, smem, stream, sweep_kernel<R, false>, c.jobs, c.passes + pass, c.ops, c.M));
+    CUDA_TRY(launch_sweep(early, grid, nt, smem, stream, sweep_kernel<R, false>, c.jobs, c.passes + pass, c.ops, c.M));
   CUDA_TRY(cudaGetLastError());
   if (c.sites && c.ps->desc[pass].has_reduce) {
     if (live) ++g_launches;
@@ -1852,6 +1893,10 @@ static LaunchCtx state_ctx(spinrp_state *st) {
   c.resident = c.resident_smem > 0;
   c.prefetch_ahead = st->prefetch_ahead;
   c.pipe_blocks = st->pipe_req ? st->pipe_blocks : 0;
+  for (int k = 0; k <= c.sites && !c.resident && !c.pipe_blocks; ++k) {  // asked for when first needed
+    if (!st->per_sm[k]) st->per_sm[k] = sweep_per_sm(st->prec, st->ps, st->plan.K, k == 1);
+    c.per_sm[k] = st->per_sm[k];
+  }
   c.pipe_err = pipe_err_word(st);
   c.segments = st->plan.segments();
   c.sweeps_per_step = st->plan.sweeps_per_step();
@@ -2960,7 +3005,8 @@ extern "C" int spinrp_batch_create(int njobs, const spinrp_system *const *system
     return rc;
   }
   for (BatchGroup &g : b->groups) {
-    if (g.ps.phased) g.ctx.prefetch_ahead = sweep2_resident(prec, g.ps.rb, g.plan.K, g.ps.oriented);
+    g.ctx.per_sm[0] = sweep_per_sm(prec, g.ps, g.plan.K, false);
+    if (g.ps.phased) g.ctx.prefetch_ahead = g.ctx.per_sm[0] * device_sms();
     g.pipe_blocks = g.ctx.resident ? 0 : pipe_grid(prec, g.plan, g.ps, g.M, (int)g.jobs.size());
     g.ctx.pipe_blocks = b->pipe_req ? g.pipe_blocks : 0;
     g.ctx.pipe_err = b->d_pipe_err;

@@ -31,7 +31,12 @@ struct LayoutArg {
 // be resident, with the pass's program staged (it does not depend on the sweep
 // before), while that sweep still runs; grid_wait() returns once every earlier
 // kernel has finished and its writes are visible, grid_go() lets the next
-// sweep's blocks in as soon as all of this one's are (see launch_sweep).
+// sweep's blocks in once all of this one's have called it (see launch_sweep).
+// A sweep calls it after its wait, so that one sweep at most waits beside the one
+// that runs: called before, the sweeps after the next came in too, and SMs filled
+// with waiting blocks got two blocks of one sweep while others had none (128-block
+// sweeps, us per step: 19-spin complex128 star 1219 -> 689, 19-spin complex64
+// chain 21.1 -> 15.9).
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -529,7 +534,6 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
   __shared__ uint64_t sOut;
   __shared__ double s_w[SITES ? kMaxWarps * kSiteSlots : 1];
   __shared__ SOp s_ops[kMaxPlainOps];
-  grid_go();
   {
     const int nwords = (int)(sizeof(PassDesc) / 4);
     for (int w = threadIdx.x; w < nwords; w += blockDim.x)
@@ -560,6 +564,7 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
     return o;
   };
   grid_wait();
+  grid_go();
   for (uint32_t t = tid; t < T; t += nt) {
     const C a = psi[base + offset(t)];
     re[t] = a.x, im[t] = a.y;
@@ -1713,7 +1718,6 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   // the tile, then the L2 prefetch of the tile of block blockIdx.x + ahead
   // (ahead = blocks resident at once): DRAM keeps streaming while tiles
   // compute, and that block's loads find its tile in L2
-  grid_go();
   {
     const char *pw = reinterpret_cast<const char *>(phases + d.phase0);
     const uint32_t a_ph = (uint32_t)__cvta_generic_to_shared(s_ph);
@@ -1725,6 +1729,7 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   }
   if (chained && d.diag) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   grid_wait();
+  grid_go();
   sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
   if constexpr (DIRECT) sw2::load_direct<RB>(psi, base, d, tid, lognt, RE, IM);
   else sw2::load_tile<RB>(psi, base, d, tid, lognt, (uint32_t)__cvta_generic_to_shared(tile2));

@@ -231,8 +231,8 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
     }
   sw2::cp_async_wait_all();
   __syncthreads();
-  grid_go();
   grid_wait();
+  grid_go();
 
   if (tid >= 2 * NT) {
     // producer: at step i write back local unit i - 3, then gather unit i

@@ -112,7 +112,6 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
   const int lognt = K - RB;
   const uint64_t base = sw2::tile_origin(blockIdx.x, d, M);
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(tile16);
-  grid_go();
   // the pass's program; FP64 coefficients from the job's table
   for (int i = tid; i < d.nphases; i += nt) s_ph[i] = phases[d.phase0 + i];
   for (int i = tid; i < d.nrops; i += nt) {
@@ -129,6 +128,7 @@ sweep2d_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ PassDes
   }
   if (d.diag) sw2::diag_fields(d, base, tid, lognt, M, jp.qdiag, sH);
   grid_wait();
+  grid_go();
   // ---- global -> shared: 16-byte async copies, amplitude a = tid + nt * e,
   // e in Gray-code order in runs of eight (as in the complex64 kernel)
   {
