@@ -319,9 +319,9 @@ int spinrp_state_orientation(const spinrp_state *st, uint64_t *black);
  * one-tile-per-block sweep; the amplitudes and series are the same bit for
  * bit.  Takes effect at the next evolve.  Host only.  Errors: SPINRP_EINVAL.
  * The pipeline's hand-over waits are bounded (2 s each); one that gives up
- * records NaN for that step's P and norm and sets the state's error word,
- * which spinrp_polarization (site 1) and spinrp_norm_series then report as
- * SPINRP_ETIMEOUT. */
+ * records NaN for that step's P (of every spin read out) and norm and sets the
+ * state's error word, which spinrp_polarization, spinrp_site_series and
+ * spinrp_norm_series then report as SPINRP_ETIMEOUT. */
 int spinrp_state_set_pipeline(spinrp_state *st, int on);
 
 /* *on = 1 when the state's sweeps run pipelined (the setting is on and the

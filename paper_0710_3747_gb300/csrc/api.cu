@@ -1392,7 +1392,7 @@ static int record_sites0(spinrp_state *st) {
   else
     state_sites_kernel<double><<<blocks, 256, 0, st->stream>>>(st->d_job, st->M, layout_arg(st));
   CUDA_TRY(cudaGetLastError());
-  sites_finalize_kernel<<<st->M, 256, 0, st->stream>>>(st->d_job, st->M, blocks);
+  sites_finalize_kernel<<<st->M, 256, 0, st->stream>>>(st->d_job, st->M, blocks, nullptr);
   CUDA_TRY(cudaGetLastError());
   return SPINRP_OK;
 }
@@ -1737,7 +1737,8 @@ static int launch_pass(const LaunchCtx &c, int pass, cudaStream_t stream, bool l
   CUDA_TRY(cudaGetLastError());
   if (c.sites && c.ps->desc[pass].has_reduce) {
     if (live) ++g_launches;
-    sites_finalize_kernel<<<dim3(c.M, c.njobs), 256, 0, stream>>>(c.jobs, c.M, 1 << (c.M - K));
+    sites_finalize_kernel<<<dim3(c.M, c.njobs), 256, 0, stream>>>(c.jobs, c.M, 1 << (c.M - K),
+                                                                  c.pipe_blocks ? c.pipe_err : nullptr);
     CUDA_TRY(cudaGetLastError());
   }
   if (live && c.prof) prof_mark(c.prof, SPINRP_KERNEL_SWEEP);
@@ -1961,24 +1962,32 @@ extern "C" int spinrp_evolve(spinrp_state *st, double dt, int64_t steps, int ord
 
 extern "C" int64_t spinrp_series_length(const spinrp_state *st) { return st ? st->len : 0; }
 
+// n doubles of a device series to the host, with the pipelined sweeps' error
+// word: a sweep whose wait gave up recorded NaN and set it.
+static int read_series(spinrp_state *st, double *dst, const double *src, int64_t n, int *perr) {
+  CUDA_TRY(cudaMemcpyAsync(dst, src, sizeof(double) * n, cudaMemcpyDeviceToHost, st->stream));
+  st->d2h += (int64_t)sizeof(double) * n;
+  if (st->pipe_blocks) {
+    CUDA_TRY(cudaMemcpyAsync(perr, pipe_err_word(st), sizeof *perr, cudaMemcpyDeviceToHost, st->stream));
+    st->d2h += (int64_t)sizeof *perr;
+  }
+  CUDA_TRY(cudaStreamSynchronize(st->stream));
+  return SPINRP_OK;
+}
+static int series_status(int perr) {
+  return perr ? fail(SPINRP_ETIMEOUT, "series: a wait of the pipelined sweep gave up") : SPINRP_OK;
+}
+
 static int copy_series(spinrp_state *st, int which, double *out, int64_t cap, int64_t *n) {
   if (!st || !n || (cap > 0 && !out)) return fail(SPINRP_EINVAL, "series: bad argument");
   *n = st->len;
   const int64_t m = std::min(cap, st->len);
   if (m <= 0) return SPINRP_OK;
   std::vector<double> buf(2 * m);
-  CUDA_TRY(cudaMemcpyAsync(buf.data(), st->series, sizeof(double) * 2 * m, cudaMemcpyDeviceToHost, st->stream));
-  st->d2h += (int64_t)sizeof(double) * 2 * m;
-  // a pipelined sweep whose wait gave up recorded NaN and set the error word
   int perr = 0;
-  if (st->pipe_blocks) {
-    CUDA_TRY(cudaMemcpyAsync(&perr, pipe_err_word(st), sizeof perr, cudaMemcpyDeviceToHost, st->stream));
-    st->d2h += (int64_t)sizeof perr;
-  }
-  CUDA_TRY(cudaStreamSynchronize(st->stream));
+  if (int rc = read_series(st, buf.data(), st->series, 2 * m, &perr)) return rc;
   for (int64_t k = 0; k < m; ++k) out[k] = buf[2 * k + which];
-  if (perr) return fail(SPINRP_ETIMEOUT, "series: a wait of the pipelined sweep gave up");
-  return SPINRP_OK;
+  return series_status(perr);
 }
 
 extern "C" int spinrp_state_set_sites(spinrp_state *st, int all_sites) {
@@ -1994,11 +2003,9 @@ extern "C" int spinrp_site_series(spinrp_state *st, double *out, int64_t cap, in
   *n = st->len;
   const int64_t m = std::min(cap, st->len);
   if (m <= 0) return SPINRP_OK;
-  CUDA_TRY(cudaMemcpyAsync(out, st->site_series, sizeof(double) * st->M * m, cudaMemcpyDeviceToHost,
-                           st->stream));
-  st->d2h += (int64_t)sizeof(double) * st->M * m;
-  CUDA_TRY(cudaStreamSynchronize(st->stream));
-  return SPINRP_OK;
+  int perr = 0;
+  if (int rc = read_series(st, out, st->site_series, st->M * m, &perr)) return rc;
+  return series_status(perr);
 }
 
 extern "C" int spinrp_polarization(spinrp_state *st, int site, double *out, int64_t cap, int64_t *n) {
@@ -2012,12 +2019,10 @@ extern "C" int spinrp_polarization(spinrp_state *st, int site, double *out, int6
   const int64_t m = std::min(cap, st->len);
   if (m <= 0) return SPINRP_OK;
   std::vector<double> buf((size_t)st->M * m);
-  CUDA_TRY(cudaMemcpyAsync(buf.data(), st->site_series, sizeof(double) * buf.size(), cudaMemcpyDeviceToHost,
-                           st->stream));
-  st->d2h += (int64_t)sizeof(double) * buf.size();
-  CUDA_TRY(cudaStreamSynchronize(st->stream));
+  int perr = 0;
+  if (int rc = read_series(st, buf.data(), st->site_series, (int64_t)buf.size(), &perr)) return rc;
   for (int64_t k = 0; k < m; ++k) out[k] = buf[k * st->M + (site - 1)];
-  return SPINRP_OK;
+  return series_status(perr);
 }
 
 extern "C" int spinrp_norm_series(spinrp_state *st, double *out, int64_t cap, int64_t *n) {

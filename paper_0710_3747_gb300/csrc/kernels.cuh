@@ -232,9 +232,10 @@ state_sites_kernel(const JobPtrs *__restrict__ jobs, int M, LayoutArg lay) {
 
 // P of every spin for the entry the preceding reduction recorded (slot
 // *step - 1): block q sums columns 0 and 1 + q over the nblk block rows in a
-// fixed order, P_q = (2 N_up - N) / N.
+// fixed order, P_q = (2 N_up - N) / N; NaN, as P and the norm, when err (if any)
+// says that a wait of the pipelined sweep gave up, which leaves columns unwritten.
 __global__ void __launch_bounds__(256)
-sites_finalize_kernel(const JobPtrs *__restrict__ jobs, int M, int nblk) {
+sites_finalize_kernel(const JobPtrs *__restrict__ jobs, int M, int nblk, const int *err) {
   const JobPtrs jp = jobs[blockIdx.y];
   const int q = blockIdx.x;
   const double *__restrict__ c0 = jp.psites;
@@ -251,7 +252,8 @@ sites_finalize_kernel(const JobPtrs *__restrict__ jobs, int M, int nblk) {
   }
   if (threadIdx.x == 0) {
     const int64_t slot = *jp.step - 1;
-    jp.site_series[slot * M + q] = (2.0 * su[0] - sn[0]) / sn[0];
+    const bool bad = err && *err != 0;
+    jp.site_series[slot * M + q] = bad ? __longlong_as_double(0x7ff8000000000000ll) : (2.0 * su[0] - sn[0]) / sn[0];
   }
 }
 
