@@ -246,6 +246,43 @@ struct PhaseState {
   int pre = 0;               // gates before the fence done
   int parent = -1;           // index into the previous beam level
   uint32_t set = 0;          // register set that produced this state
+  int penalty = 0;           // among states of as many gates done, the least first
+};
+
+// The bits' gate chains in one array, each ended by -1, for the closures of the
+// beam search (a few thousand per phase): only what a set reaches, not in which
+// order, so the gates of a bit are taken as far as they go.
+struct Chains {
+  std::vector<int> flat, ends;  // chain of bit q from flat[off[q]]; sum of a gate's two bits
+  std::array<int, kMaxK> off{};
+  Chains(const std::vector<std::pair<int, int>> &g, const std::vector<std::vector<int>> &chain) {
+    for (int q = 0; q < (int)chain.size(); ++q) {
+      off[q] = (int)flat.size();
+      flat.insert(flat.end(), chain[q].begin(), chain[q].end());
+      flat.push_back(-1);
+    }
+    for (const auto &e : g) ends.push_back(e.first + e.second);
+  }
+  // what phase_closure does, without the list of gates
+  int closure(BitPtr &ptr, uint32_t R, int fence, int *pre) const {
+    int applied = 0;
+    for (bool progress = true; progress;) {
+      progress = false;
+      for (uint32_t m = R; m; m &= m - 1u) {
+        const int q = __builtin_ctz(m);
+        for (;;) {
+          const int b = flat[off[q] + ptr[q]];
+          if (b < 0 || (b >= fence && *pre != fence)) break;
+          const int o = ends[b] - q;
+          if (!((R >> o) & 1u) || flat[off[o] + ptr[o]] != b) break;
+          ++ptr[q], ++ptr[o], ++applied;
+          if (b < fence) ++*pre;
+          progress = true;
+        }
+      }
+    }
+    return applied;
+  }
 };
 
 // Apply every gate reachable inside bit set R (smallest index first); gates
@@ -315,6 +352,7 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
     chain[gates[b].first].push_back(b);
     chain[gates[b].second].push_back(b);
   }
+  const Chains chains(gates, chain);
   std::vector<std::vector<PhaseState>> levels(1);
   if (fence < 0 || fence > n) fence = n;
   BitPtr zero;
@@ -336,7 +374,23 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
   };
   for (int depth = 0; depth < 4 * n + 4; ++depth) {
     const std::vector<PhaseState> &cur = levels.back();
-    std::vector<PhaseState> next;
+    // the `beam` best distinct states (most gates done, then least penalty, then
+    // the first found), in that order
+    std::vector<PhaseState> kept;
+    auto before = [](const PhaseState &a, const PhaseState &b) {
+      return a.done != b.done ? a.done > b.done : a.penalty < b.penalty;
+    };
+    auto keep = [&](const PhaseState &ch) {
+      if ((int)kept.size() >= beam && !before(ch, kept.back())) return;
+      for (size_t k = 0; k < kept.size(); ++k)
+        if (kept[k].ptr == ch.ptr) {
+          if (!before(ch, kept[k])) return;
+          kept.erase(kept.begin() + k);
+          break;
+        }
+      kept.insert(std::upper_bound(kept.begin(), kept.end(), ch, before), ch);
+      if ((int)kept.size() > beam) kept.pop_back();
+    };
     for (int si = 0; si < (int)cur.size(); ++si) {
       const PhaseState &st = cur[si];
       // bits with gates still to do; a useful set holds RB of them (all of
@@ -344,13 +398,19 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
       std::vector<int> live;
       for (int q = 0; q < K; ++q)
         if (st.ptr[q] < chain[q].size()) live.push_back(q);
+      // the gates that can come next: most sets hold none of them
+      std::vector<uint32_t> ready;
+      for (int q : live) {
+        const int b = chain[q][st.ptr[q]], o = chains.ends[b] - q;
+        if (q < o && chains.flat[chains.off[o] + st.ptr[o]] == b && (b < fence || st.pre == fence))
+          ready.push_back(1u << q | 1u << o);
+      }
       auto try_set = [&](uint32_t R) {
+        if (std::none_of(ready.begin(), ready.end(), [&](uint32_t m) { return (m & ~R) == 0u; })) return;
         PhaseState ch{st.ptr, st.done, st.pre, si, R};
-        const int a = phase_closure(gates, chain, ch.ptr, R, fence, &ch.pre, nullptr);
-        if (a > 0) {
-          ch.done += a;
-          next.push_back(std::move(ch));
-        }
+        ch.done += chains.closure(ch.ptr, R, fence, &ch.pre);
+        ch.penalty = penalty(ch, depth);
+        keep(ch);
       };
       if (nb_allowed == 0) {
         // the first set holds ends.first; a set that may be the last one is
@@ -390,22 +450,7 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
         }
       }
     }
-    if (next.empty()) return false;
-    // keep the `beam` best distinct states (most gates done)
-    std::stable_sort(next.begin(), next.end(), [&](const PhaseState &a, const PhaseState &b) {
-      return a.done != b.done ? a.done > b.done : penalty(a, depth) < penalty(b, depth);
-    });
-    std::vector<PhaseState> kept;
-    for (PhaseState &c : next) {
-      bool dup = false;
-      for (const PhaseState &k : kept)
-        if (k.ptr == c.ptr) {
-          dup = true;
-          break;
-        }
-      if (!dup) kept.push_back(std::move(c));
-      if ((int)kept.size() >= beam) break;
-    }
+    if (kept.empty()) return false;
     levels.push_back(std::move(kept));
     if (levels.back().front().done == n) {
       // walk back the sets of the first finished state, then replay them
@@ -438,67 +483,80 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
 // ---------------------------------------------------------------------------
 namespace {
 
-// Rounds of gates [from, to) under the labelling ku < kv (combo: the pair's
-// index); returns their number and writes them when out is non-null.
-int greedy_rounds(const std::vector<int> &ku, const std::vector<int> &kv, const std::vector<int> &combo, int RB,
-                  int from, int to, std::vector<PhaseRound> *out) {
-  std::array<std::vector<int>, kMaxRegBits> chain;  // per register bit: its gates in order
-  std::array<size_t, kMaxRegBits> ptr{};
-  for (int g = from; g < to; ++g) chain[ku[g]].push_back(g), chain[kv[g]].push_back(g);
-  int n = 0;
-  for (int left = to - from; left > 0; ++n) {
-    PhaseRound r;
-    for (int u = 0; u < RB; ++u)
-      for (int v = u + 1; v < RB; ++v)
-        if (ptr[u] < chain[u].size() && ptr[v] < chain[v].size() && chain[u][ptr[u]] == chain[v][ptr[v]]) {
-          r.gates.push_back(chain[u][ptr[u]]);
-          ++ptr[u], ++ptr[v];
-        }
-    left -= (int)r.gates.size();
-    r.combo = combo;
-    if (out) out->push_back(r);
+// A phase's gates by register bit.
+struct RoundGates {
+  int RB, n;
+  std::vector<int> pos;     // the register bits, ascending tile bits
+  std::vector<int> ku, kv;  // a gate's two bits, as indices into pos
+  std::array<std::vector<int>, kMaxRegBits> chain;  // a bit's gates in order, then n
+  RoundGates(const std::vector<std::pair<int, int>> &gates, const std::vector<int> &rb)
+      : RB((int)rb.size()), n((int)gates.size()), pos(rb) {
+    std::sort(pos.begin(), pos.end());
+    auto at = [&](int q) { return (int)(std::find(pos.begin(), pos.end(), q) - pos.begin()); };
+    for (int g = 0; g < n; ++g) {
+      ku.push_back(at(gates[g].first)), kv.push_back(at(gates[g].second));
+      chain[ku[g]].push_back(g), chain[kv[g]].push_back(g);
+    }
+    for (int k = 0; k < RB; ++k) chain[k].push_back(n);
   }
-  return n;
-}
+  // Rounds of the gates before `split`, then of the others, with the bits in the
+  // order `order` (indices into pos): their number, or `most` if that many or
+  // more; written when out is non-null, an empty one between them for split >= 0.
+  int rounds(const std::vector<int> &order, int split, int most, std::vector<PhaseRound> *out) const {
+    std::array<int, kMaxRegBits> ptr{};
+    std::vector<int> combo;
+    if (out) {
+      std::array<int, kMaxRegBits> idx{};
+      for (int k = 0; k < RB; ++k) idx[order[k]] = k;
+      for (int g = 0; g < n; ++g) {
+        const int u = std::min(idx[ku[g]], idx[kv[g]]), v = std::max(idx[ku[g]], idx[kv[g]]);
+        combo.push_back(u * (2 * RB - u - 1) / 2 + v - u - 1);
+      }
+    }
+    int r = 0, done = 0;
+    for (int part = 0; part < 2; ++part) {
+      const int to = part ? n : std::max(split, 0);
+      while (done < to) {
+        if (r >= most) return most;
+        PhaseRound rd;
+        for (int u = 0; u < RB; ++u)
+          for (int v = u + 1; v < RB; ++v) {
+            const int a = order[u], b = order[v], g = chain[a][ptr[a]];
+            if (g >= to || g != chain[b][ptr[b]]) continue;
+            ++ptr[a], ++ptr[b], ++done;
+            if (out) rd.gates.push_back(g);
+          }
+        ++r;
+        if (out) rd.combo = combo, out->push_back(rd);
+      }
+      if (out && split >= 0 && part == 0) out->push_back(PhaseRound{});
+    }
+    return std::min(r, most);
+  }
+};
 
 }  // namespace
 
 void plan_rounds(const std::vector<std::pair<int, int>> &gates, int RB, int split, int fix1, int fix2,
                  int fix_last, std::vector<int> *rb, std::vector<PhaseRound> *rounds) {
-  const int n = (int)gates.size();
-  std::vector<int> order = *rb, best_order;  // order[k]: tile bit of register bit k
-  std::sort(order.begin(), order.end());
-  std::vector<int> ku(n), kv(n), combo(n), idx(kMaxK);
-  auto label = [&]() {
-    for (int k = 0; k < RB; ++k) idx[order[k]] = k;
-    int pack = 0;
-    for (int g = 0; g < n; ++g) {
-      const int a = idx[gates[g].first], b = idx[gates[g].second];
-      ku[g] = std::min(a, b), kv[g] = std::max(a, b);
-      combo[g] = ku[g] * (2 * RB - ku[g] - 1) / 2 + kv[g] - ku[g] - 1;
-      pack += ku[g] == 0;
-    }
-    return pack;
-  };
-  const int cut = split < 0 ? 0 : split;
+  const RoundGates rg(gates, *rb);
+  std::vector<int> order(RB), best_order;
+  for (int k = 0; k < RB; ++k) order[k] = k;
   // a gate on the pack bit costs a gate more, a round about two (its tests)
   int best = std::numeric_limits<int>::max();
   do {
-    if ((fix1 >= 0 && order[1] != fix1) || (fix2 >= 0 && order[2] != fix2) ||
-        (fix_last >= 0 && order[RB - 1] != fix_last))
+    if ((fix1 >= 0 && rg.pos[order[1]] != fix1) || (fix2 >= 0 && rg.pos[order[2]] != fix2) ||
+        (fix_last >= 0 && rg.pos[order[RB - 1]] != fix_last))
       continue;
-    const int pack = label();
+    const int pack = (int)rg.chain[order[0]].size() - 1;
     if (pack >= best) continue;
-    const int r = greedy_rounds(ku, kv, combo, RB, 0, cut, nullptr) + greedy_rounds(ku, kv, combo, RB, cut, n, nullptr);
-    if (pack + 2 * r < best) best = pack + 2 * r, best_order = order;
+    const int most = best == std::numeric_limits<int>::max() ? best : (best - pack + 1) / 2;
+    const int r = rg.rounds(order, split, most, nullptr);
+    if (r < most) best = pack + 2 * r, best_order = order;
   } while (std::next_permutation(order.begin(), order.end()));
-  order = best_order;
-  label();
-  *rb = order;
+  for (int k = 0; k < RB; ++k) (*rb)[k] = rg.pos[best_order[k]];
   rounds->clear();
-  greedy_rounds(ku, kv, combo, RB, 0, cut, rounds);
-  if (split >= 0) rounds->push_back(PhaseRound{});
-  greedy_rounds(ku, kv, combo, RB, cut, n, rounds);
+  rg.rounds(best_order, split, std::numeric_limits<int>::max(), rounds);
 }
 
 }  // namespace spinrp
