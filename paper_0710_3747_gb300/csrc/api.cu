@@ -715,14 +715,9 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
       std::vector<ROp> pending;  // element-wise ops waiting for the next phase
       d.direct = want_direct;
       // lanes: bits that should be lane bits if they are not in registers
-      auto new_phase = [&](std::vector<int> rb, const std::vector<int> &prefer = {}) {
+      auto new_phase = [&](const std::vector<int> &rb, const std::vector<int> &prefer = {}) {
         PhaseDesc ph;
         memset(&ph, 0, sizeof ph);
-        // a readout without gates: its spin on the last register bit
-        for (const ROp &r : pending)
-          if (rounds && r.kind == OP_REDUCE)
-            for (int k = 0; k < RB; ++k)
-              if (rb[k] == d.site_tile) std::swap(rb[k], rb[RB - 1]);
         uint32_t isreg = 0;
         for (int k = 0; k < RB; ++k) ph.rb[k] = (uint8_t)rb[k], isreg |= 1u << rb[k];
         // lane bits: nres non-register bits of distinct residues mod nres
@@ -752,6 +747,17 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
         pending.clear();
         ps->phases.push_back(ph);
         d.nphases++;
+      };
+      // a phase of the pending ops alone; a readout's spin on the last register bit
+      auto readout_pending = [&] {
+        return rounds && std::any_of(pending.begin(), pending.end(), [](const ROp &r) { return r.kind == OP_REDUCE; });
+      };
+      auto idle_phase = [&] {
+        std::vector<int> rb = default_rb;
+        if (readout_pending())
+          for (int k = 0; k < RB; ++k)
+            if (rb[k] == d.site_tile) std::swap(rb[k], rb[RB - 1]);
+        new_phase(rb);
       };
       auto push_rop = [&](const ROp &r) {
         ps->rops.push_back(r);
@@ -816,7 +822,8 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
             const bool first = first_of && k == 0, last = last_of && k + 1 == sets.size();
             const int fix1 = last ? d.perm[0] : first ? 0 : -1, fix2 = last ? d.perm[1] : first ? 1 : -1;
             // the readout spin on the last register bit, unless it is a fixed one
-            const bool hold = split >= 0 && d.site_tile >= 0 && ((sets[k] >> d.site_tile) & 1) &&
+            const bool reads = split >= 0 || (k == 0 && readout_pending());
+            const bool hold = reads && d.site_tile >= 0 && ((sets[k] >> d.site_tile) & 1) &&
                               d.site_tile != fix1 && d.site_tile != fix2;
             plan_rounds(pg, RB, split, fix1, fix2, hold ? d.site_tile : -1, &rb, &rounds_of);
             if (last) new_phase(rb, {d.perm[2], d.perm[3]});
@@ -905,9 +912,9 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
         if (!flush(gates, false)) return false;
         if (op.kind == OP_DIAG) {
           // the diagonal phase runs alone (its own phase, no register subcube)
-          if (!pending.empty()) new_phase(default_rb);
+          if (!pending.empty()) idle_phase();
           pending.push_back(r);
-          new_phase(default_rb);
+          idle_phase();
           last_is_diag = true;
         } else if (d.nphases > 0 && pending.empty() && !last_is_diag) {
           push_rop(r);
@@ -916,7 +923,7 @@ static bool compile_phases(PassSet *ps, int M, int K, int RB, int prec, std::str
         }
       }
       if (!flush(gates, true)) return false;
-      if (!pending.empty() || d.nphases == 0) new_phase(default_rb), d.direct = 0;
+      if (!pending.empty() || d.nphases == 0) idle_phase(), d.direct = 0;
       if (d.direct) {
         const PhaseDesc &a = ps->phases[d.phase0], &b = ps->phases.back();
         std::vector<int> out(K);  // output tile bit of each input tile bit
