@@ -152,10 +152,19 @@ def flipflop(psi: np.ndarray, i: int, j: int, b: float, tau: float, threads: int
     lib().oracle_flipflop(M, _dptr(_as_buf(psi)), i, j, float(b), float(tau), _threads(threads))
 
 
+def _of_state(a: np.ndarray, M: int) -> np.ndarray:
+    """The M x M coupling matrix of a state of M spins from one of the first spins;
+    the others are uncoupled."""
+    a = np.asarray(a, dtype=np.float64)
+    if a.ndim != 2 or a.shape[0] != a.shape[1] or a.shape[0] > M:
+        raise ValueError(f"couplings of shape {a.shape} for a state of {M} spins")
+    return np.ascontiguousarray(np.pad(a, (0, M - a.shape[0])))
+
+
 def diag(psi: np.ndarray, a: np.ndarray, tau: float, threads: int | None = None):
     """In place: exp(-i tau sum_{i<j} a_ij S^z_i S^z_j)."""
     M = int(np.log2(psi.size))
-    a = np.ascontiguousarray(a, dtype=np.float64)
+    a = _of_state(a, M)
     lib().oracle_diag(M, _dptr(_as_buf(psi)), _dptr(a), float(tau), _threads(threads))
 
 
@@ -197,8 +206,7 @@ def evolve(psi: np.ndarray, a: np.ndarray, b: np.ndarray, dt: float, steps: int,
     and the norm after each step.
     """
     M = int(np.log2(psi.size))
-    a = np.ascontiguousarray(a, dtype=np.float64)
-    b = np.ascontiguousarray(b, dtype=np.float64)
+    a, b = _of_state(a, M), _of_state(b, M)
     if bonds is None:
         bonds = canonical_bonds(b)
     bl = np.ascontiguousarray(np.asarray(list(bonds), dtype=np.int32).reshape(-1, 2))
@@ -270,8 +278,7 @@ def evolve_all_sites(psi: np.ndarray, a: np.ndarray, b: np.ndarray, dt: float, s
                                           ctypes.c_int]
     L.oracle_evolve_all_sites.restype = ctypes.c_int
     M = int(np.log2(psi.size))
-    a = np.ascontiguousarray(a, dtype=np.float64)
-    b = np.ascontiguousarray(b, dtype=np.float64)
+    a, b = _of_state(a, M), _of_state(b, M)
     if bonds is None:
         bonds = canonical_bonds(b)
     bl = np.ascontiguousarray(np.asarray(list(bonds), dtype=np.int32).reshape(-1, 2))
