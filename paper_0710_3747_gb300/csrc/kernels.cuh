@@ -514,11 +514,14 @@ __device__ __forceinline__ void shear_plane(double &x, double &y, double t, doub
 // op and coefficients read from global memory at each gate and both planes in
 // one thread, 0.45 us so (the 26-gate sweep 23 -> 18 us with its launch, the
 // 400-step job 15.0 -> 10.3 ms with the sweeps chained too).
+// Two blocks of 512 threads share an SM, so 64 registers: the readout keeps five
+// sums for the bits a thread walks, not one for every tile bit, which took 86 and
+// an SM a block at a time (20-spin complex128 all-site chain 246 -> 208 us a step).
 constexpr int kMaxPlainOps = 192;  // every pair of 14 tile bits twice, and the element-wise ops
 static_assert(kMaxK * (kMaxK - 1) + 4 <= kMaxPlainOps, "ops of a pass");
 
 template <typename R, bool SITES>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(512, 2)
 sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdesc,
              const Op *__restrict__ ops, int M) {
   using C = typename CT<R>::T;
@@ -644,9 +647,10 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
       }
       __syncthreads();
     } else if (op.kind == OP_REDUCE) {
-      R tsum = 0, uhi[kMaxK];
+      // weights by the tile bits a thread walks, L and up (L is nine, or K - 1 or K below that)
+      R tsum = 0, uhi[kMaxK - 9];
 #pragma unroll
-      for (int q = 0; q < kMaxK; ++q) uhi[q] = 0;
+      for (int e = 0; e < kMaxK - 9; ++e) uhi[e] = 0;
       for (uint32_t t = tid; t < T; t += nt) {
         const R pr = re[t] * re[t] + im[t] * im[t];
         const uint64_t bit = d.site_tile >= 0 ? ((t >> d.site_tile) & 1u)
@@ -656,15 +660,16 @@ sweep_kernel(const JobPtrs *__restrict__ jobs, const PassDesc *__restrict__ pdes
         if constexpr (SITES) {
           tsum += pr;
 #pragma unroll
-          for (int q = 0; q < kMaxK; ++q)
-            if (q >= L && q < K && ((t >> q) & 1u)) uhi[q] += pr;
+          for (int e = 0; e < kMaxK - 9; ++e)
+            if ((t >> (L + e)) & 1u) uhi[e] += pr;
         }
       }
       if constexpr (SITES) {
         // tile bits below L come from the thread index: the thread's whole sum
 #pragma unroll
         for (int q = 0; q < kMaxK; ++q)
-          warp_site_sum<R>(q < L ? (((tid >> q) & 1) ? tsum : (R)0) : uhi[q], q, s_w, tid);
+          warp_site_sum<R>(q < L ? (((tid >> q) & 1) ? tsum : (R)0) : q == L ? uhi[0] : q > 9 ? uhi[q - 9] : (R)0,
+                           q, s_w, tid);
         warp_site_sum<R>(tsum, kMaxK, s_w, tid);
       }
       __syncthreads();  // later ops overwrite the tile
