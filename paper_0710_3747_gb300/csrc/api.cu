@@ -299,11 +299,12 @@ extern "C" int spinrp_system_set_regbits(spinrp_system *sys, int rb) {
 // of 14 spins 14.9 / 19.0 / 16.0, 18 18.5 / 22.9 / 34.4, 22 87.9 / 63.6 / 80.2,
 // 24 306.5 / 296.7 / 278.0, 26 1172 / 1069 / 1397; dipolar stars of 16 45.6 /
 // 58.7 / 90.4, 20 106.6 / 139.2 / 125.9, 22 358.5 / 318.3 / 363.4, 24 1421 /
-// 1339 / 1436 (the model's pick is the fastest but on the 24-spin ladder, 6 %).  Where 13-spin tiles run as the pipelined sweep
-// (pipe_kernel: six register bits, plain storage, at least four units per
-// SM) a sweep costs kPipeSweepCost of the model's sweep: per-sweep time measured
-// (before the register programs' walks) of the pipelined 13-spin sweep over the 14-spin one 0.58, 0.59 and
-// 0.72 on dipolar stars of 23, 24 and 26 spins, 0.48, 0.70 and 0.67 on
+// 1339 / 1436 (the model's pick is the fastest but on the 24-spin ladder, 6 %).
+// Where 13-spin tiles run as the pipelined sweep (pipe_kernel: six register
+// bits, plain storage, at least four units per SM) a sweep costs kPipeSweepCost
+// of the model's sweep: per-sweep time measured (before the register programs'
+// walks) of the pipelined 13-spin sweep over the 14-spin one 0.58, 0.59 and 0.72
+// on dipolar stars of 23, 24 and 26 spins, 0.48, 0.70 and 0.67 on
 // ladders of 24, 26 and 28 spins, 0.49 and 0.47 on batches of 383 and 363
 // dipolar stars of 20 and 21 spins (8 sweeps per step against 4: 29.2
 // against 30.0 and 57.8 against 62.2 ms per step); with 0.5 the model picks
@@ -1221,8 +1222,8 @@ static unsigned pipe_grid(int prec, const Plan &plan, const PassSet &ps, int M, 
   int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pipe_kernel<6, 13, false, kPipeDiag>, kPipeThreads, kPipeSmem) !=
-          cudaSuccess) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, pipe_kernel<6, 13, false, kPipeDiag>, kPipeThreads,
+                                                    kPipeSmem) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -2955,7 +2956,8 @@ extern "C" int spinrp_batch_create(int njobs, const spinrp_system *const *system
       if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);  // bv/am are reused
       b->hjobs[g.jobs[k]] = p;
     }
-    if (e == cudaSuccess && (e = up(d + o_pass, g.ps.desc.data(), sizeof(PassDesc) * g.ps.desc.size())) == cudaSuccess &&
+    if (e == cudaSuccess &&
+        (e = up(d + o_pass, g.ps.desc.data(), sizeof(PassDesc) * g.ps.desc.size())) == cudaSuccess &&
         (e = up(d + o_ops, g.ps.ops.data(), sizeof(Op) * g.ps.ops.size())) == cudaSuccess &&
         (e = up(d + o_ph, g.ps.phases.data(), sizeof(PhaseDesc) * g.ps.phases.size())) == cudaSuccess &&
         (e = up(d + o_rop, g.ps.rops.data(), sizeof(ROp) * g.ps.rops.size())) == cudaSuccess &&

@@ -242,8 +242,9 @@ bool plan_phases(int K, const std::vector<std::pair<int, int>> &gates, int RB, i
 // Rounds of one phase's gates (pairs of tile bits, in order): chooses the order
 // of the RB register bits in *rb (bit 0 is the pack bit, whose gates are
 // scalar) and cuts the gates into rounds, walks over the register-bit pairs in
-// lexicographic order that keep every bit's gate sequence, for few rounds and few gates on the pack bit.  An empty round
-// stands for the readout after the first `split` gates (split < 0: none).
+// lexicographic order that keep every bit's gate sequence, for few rounds and few
+// gates on the pack bit.  An empty round stands for the readout after the first
+// `split` gates (split < 0: none).
 // fix1, fix2, fix_last: tile bits that register bits 1, 2 and RB - 1 hold (-1: any).
 struct PhaseRound {
   std::vector<int> gates;  // indices into the phase's gates, in execution order

@@ -905,18 +905,20 @@ __device__ __forceinline__ void gate_combo(u64 (&RE)[32], u64 (&IM)[32], int com
     default: gate_of<32, 14>(RE, IM, t, s); break;
   }
 }
-__device__ __forceinline__ void gate_combo(u64 (&)[16], u64 (&)[16], int, float, float) {}  // walks only
 
 // One round of a phase's gates: the pairs of `mask` in ascending order of C,
 // coefficients from consecutive ops.  Straight code with a test before each
 // pair: gates that run follow each other in the instruction stream, and the
 // next gate's coefficients load while this one computes.  A jump per gate (a
 // switch on the pair) took about 280 cycles a gate for a lone warp, most of it
-// the jump and the instruction fetch after it; this takes about 57 (a six-gate
-// phase of a 2^12 tile 2850 -> 1890 cycles).  One walk direction only: with a second, descending copy the sweep's code outgrew the
-// instruction cache (stalls on instructions 1.7 per issue against 0.3, 15 %
-// slower on ladders); the phase planner orders the register bits so that one
-// ascending walk takes nearly every phase.
+// the jump and the instruction fetch after it; a walk takes about 320 cycles and
+// 57 a gate (clock64 around it in resident_kernel, five register bits: 519 cycles
+// for 3.6 gates on the 10-spin ladder, 649 for 5.7 on the 12-spin star; a six-gate
+// phase of a 2^12 tile 2850 -> 1890).  One walk direction only: with a second,
+// descending copy the sweep's code outgrew the instruction cache (stalls on
+// instructions 1.7 per issue against 0.3, 15 % slower on ladders); the phase
+// planner orders the register bits so that one ascending walk takes nearly every
+// phase.
 template <int NP, int C = 0>
 __device__ __forceinline__ void run_round(u64 (&RE)[NP], u64 (&IM)[NP], uint32_t mask, const ROpRes *op, float2 ts) {
   constexpr int RB = NP == 16 ? 5 : 6, NC = RB * (RB - 1) / 2;
@@ -942,9 +944,6 @@ __host__ __device__ constexpr bool gray_up(int g) { return (((g ^ (g >> 1)) >> c
 // move an amplitude pair to an odd slot, so 16-byte copies would misalign.
 __device__ __forceinline__ void cp_async8(uint32_t smem_addr, const void *gmem) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async4(uint32_t smem_addr, const void *gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async16(uint32_t smem_addr, const void *gmem) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr), "l"(gmem) : "memory");
@@ -1531,7 +1530,8 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
     // the phase's first step, and the coefficients of its first gate if it is a round
     uint32_t step = ORIENT ? 0u : d.steps[st];
     if (DIAG && (ORIENT ? ph.nops == 1 && s_op[o0].kind == OP_DIAG : (step & kStepDiag) != 0)) {
-      diag_tile<RB, ORIENT>(tile2, dtab + s_op[o0].tab, sH + s_op[o0].arg * kFieldStride, d.K, tid, lognt, d.black_tile, outer_par);
+      diag_tile<RB, ORIENT>(tile2, dtab + s_op[o0].tab, sH + s_op[o0].arg * kFieldStride, d.K, tid, lognt,
+                            d.black_tile, outer_par);
       sync();
       ++st;
       continue;
@@ -1576,6 +1576,7 @@ __device__ __forceinline__ void run_phases(float2 *tile2, const PassDesc &d, con
         if constexpr (WALK) {
           run_round<NP>(RE, IM, step & 0x7fffu, s_op + k + 1, ts);
         } else {
+          static_assert(WALK || ORIENT || RB == 6, "a jump to each gate: six register bits");
           for (int i = 1; i <= n; ++i) {
             const ROpRes cur = s_op[k + i];
             gate_combo(RE, IM, cur.combo, cur.t, cur.s);
@@ -1747,8 +1748,8 @@ sweep2_kernel(const JobPtrs *__restrict__ jobs, float2 *psi1, const ROpRes *sops
   __syncthreads();
 
   float up = 0.f, dn = 0.f;
-  sw2::run_phases<RB, SITES, ORIENT, DIRECT ? sw2::kDirect : sw2::kInPlace>(tile2, d, s_ph, s_op, base, tid, lognt, jp.dtab, up, dn, sH, s_w,
-                                             sw2::SyncBlock{}, RE, IM, psi);
+  sw2::run_phases<RB, SITES, ORIENT, DIRECT ? sw2::kDirect : sw2::kInPlace>(
+      tile2, d, s_ph, s_op, base, tid, lognt, jp.dtab, up, dn, sH, s_w, sw2::SyncBlock{}, RE, IM, psi);
   if constexpr (!DIRECT) sw2::store_tile<RB>(psi, base, d, tid, lognt, tile2);
   if constexpr (SITES)
     if (d.has_reduce) write_site_partials(d, M, base, s_w, jp.psites, tid, nt, blockIdx.x, gridDim.x);
@@ -1803,8 +1804,8 @@ resident_kernel(const JobPtrs *__restrict__ jobs, const __grid_constant__ Reside
     const PassDesc &d = steps == 1 ? rp.only : k == 0 ? rp.first : k == steps - 1 ? rp.last : rp.mid;
     float up = 0.f, dn = 0.f;
     sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
-    sw2::run_phases<RB, false, ORIENT, sw2::kInPlace>(tile2, d, s_ph + d.phase0, s_op + d.rop0, 0ull, tid, lognt, jp.dtab,
-                                              up, dn, sH, nullptr, sw2::SyncBlock{}, RE, IM, nullptr);
+    sw2::run_phases<RB, false, ORIENT, sw2::kInPlace>(tile2, d, s_ph + d.phase0, s_op + d.rop0, 0ull, tid, lognt,
+                                                      jp.dtab, up, dn, sH, nullptr, sw2::SyncBlock{}, RE, IM, nullptr);
     // this step's N_up / N_dn: FP64 sums over the block in a fixed order
     double u = up, w = dn;
     for (int o = 16; o; o >>= 1) {

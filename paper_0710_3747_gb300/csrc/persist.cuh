@@ -278,8 +278,8 @@ persist_kernel(const PersistPlan *__restrict__ plan, unsigned long long *queue, 
     __syncthreads();
     float up = 0.f, dn = 0.f;
     sw2::u64 RE[1 << (RB - 1)], IM[1 << (RB - 1)];
-    sw2::run_phases<RB, false, false, sw2::kInPlace>(tile2, d, s_ph, s_op, base, tid, lognt, jp.dtab, up, dn, sH, nullptr,
-                                             sw2::SyncBlock{}, RE, IM, nullptr);
+    sw2::run_phases<RB, false, false, sw2::kInPlace>(tile2, d, s_ph, s_op, base, tid, lognt, jp.dtab, up, dn, sH,
+                                                     nullptr, sw2::SyncBlock{}, RE, IM, nullptr);
     sw2::store_tile<RB>(psi, base, d, tid, lognt, tile2);
     if (d.has_reduce) pq::reduce_tile((double)up, (double)dn, jp, r, G.tiles, s_up, s_dn, &s_last);
     __threadfence();

@@ -17,7 +17,8 @@
 // one warp of every warpgroup.  The block is launched at 168 registers a
 // thread (3 x 128 x 168 = 64512); the producer gives registers back
 // (setmaxnreg.dec to 56) and the compute groups take them (setmaxnreg.inc to
-// 224, what the phases need without spilling): 128 x 56 + 256 x 224 = 64512.
+// 224): 128 x 56 + 256 x 224 = 64512.  The phases fit but for 8 to 40 bytes of
+// spill stores a variant.
 //
 // Three tile buffers rotate through load -> phases -> store.  Block b takes
 // the units b, b + G, b + 2G, ... (G blocks; a unit is a tile, or for a batch
@@ -155,8 +156,8 @@ __device__ __forceinline__ void pipe_finalize(const double2 *partials, unsigned 
 // group.
 //   BATCH = false: one job; jobs[0] holds its pointers (gate tables,
 //     partials, ticket, series), psi1, sops1, qdiag1 and dtab1 its amplitudes,
-//     resolved ops and diagonal-phase tables; the units are its tiles, and the last block to finish combines
-//     the tile partials.
+//     resolved ops and diagonal-phase tables; the units are its tiles, and the
+//     last block to finish combines the tile partials.
 //   BATCH = true: njobs jobs of the same plan (jobs[j]), job j's amplitudes,
 //     resolved ops and tables at those addresses plus j x jstride bytes; the units
 //     are the (job, tile) pairs, job-major; the producer copies each unit's job
@@ -173,9 +174,12 @@ __device__ __forceinline__ void pipe_finalize(const double2 *partials, unsigned 
 // few (kPipeSparse: a jump to each gate's code; most pairs of a walk would be
 // skipped, and the whole walk's code competes for the instruction cache with
 // the producer's).  kPipeSites: a reducing pass that takes the all-site readout,
-// with or without the diagonal op.  Measured with walks against jumps: 25-spin dipolar star
-// (8.7 gates a phase) 18.3 against 21.8 ms for six steps, 26-spin ladder (5.4)
-// 24.5 against 22.5 ms for twenty; the line lies between.
+// with or without the diagonal op.  Walks against jumps, us per step, by gates a
+// phase: 24-spin star 9.1 1192 / 1377; 23-spin random graphs 7.6 528 / 593, 6.2
+// 367 / 390, 5.3 252 / 261, 4.1 88.3 / 86.5; ladders 5.4..5.6, 24 spins 294 / 296,
+// 26 1083 / 1086, 30 (six steps and the initial state) 115.6 / 113.8 ms.  The
+// line is the one that keeps large ladders on jumps with room; graphs of 5 to 7
+// gates a phase would gain up to 6 % from walks.
 constexpr int kPipeDenseGates = 7;
 enum { kPipeSparse = 0, kPipeDense = 1, kPipeDiag = 2, kPipeSites = 3 };
 constexpr int kPipeBatchOps = kMaxPassOps / 3;  // resolved ops of a pass, per buffer (batches)
@@ -184,7 +188,8 @@ static_assert(sizeof(JobPtrs) % 8 == 0, "job pointers copied as 8-byte words");
 template <int RB, int K, bool BATCH, int VAR>
 __global__ void __launch_bounds__(kPipeThreads, 1)
 pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROpRes *sops1,
-            const uint64_t *qdiag1, const uint64_t *dtab1, long long jstride, const __grid_constant__ PassDesc d, const PhaseDesc *__restrict__ phases, int M, int *err, int probe) {
+            const uint64_t *qdiag1, const uint64_t *dtab1, long long jstride, const __grid_constant__ PassDesc d,
+            const PhaseDesc *__restrict__ phases, int M, int *err, int probe) {
   constexpr int LOGNT = K - RB;
   constexpr int NT = 1 << LOGNT;   // threads of a group (a warpgroup)
   constexpr int NW = NT / 32;      // warps of a group
@@ -262,7 +267,8 @@ pipe_kernel(const JobPtrs *__restrict__ jobs, int njobs, float2 *psi1, const ROp
           // the unit's job pointers and ops beside its tile
           const JobPtrs *src = jobs + (u >> lt);
           if (pt < (int)(sizeof(JobPtrs) / 8))
-            sw2::cp_async8(a_jobs + (uint32_t)sizeof(JobPtrs) * b + 8u * pt, reinterpret_cast<const char *>(src) + 8 * pt);
+            sw2::cp_async8(a_jobs + (uint32_t)sizeof(JobPtrs) * b + 8u * pt,
+                           reinterpret_cast<const char *>(src) + 8 * pt);
           const ROpRes *so =
               reinterpret_cast<const ROpRes *>(reinterpret_cast<const char *>(sops1) + (long long)(u >> lt) * jstride) +
               d.rop0;

@@ -2,7 +2,8 @@
 //
 // The complex128 counterpart of sweep2_kernel: the same pass programs (phases
 // of register bits, gates as three shears per plane, the tabulated diagonal op,
-// the fused P/norm readout), with 32 FP64 amplitudes per thread and 16-byte shared-memory slots.  Bound by the FP64 pipe.
+// the fused P/norm readout), with 32 FP64 amplitudes per thread and 16-byte
+// shared-memory slots.  Bound by the FP64 pipe.
 #pragma once
 #include "kernels.cuh"
 
